@@ -42,7 +42,7 @@ struct DevPop {
     uint8_t* arena;      // nbuf * cap bytes
     uint32_t* buf;       // [P] buffer holding individual i
     uint32_t* size;      // [P]
-    float* x;            // [Cpad] (padded cases are 0; integer set: int32 bits; Boolean: unused)
+    float* x;            // [Cpad] (padded cases repeat the last; integer set: int32 bits; Boolean: unused)
     float* t;            // [C] targets (integer set: int32 bits; Boolean: the target's case words)
     float* consts;       // [251] (integer set: int32 bits)
     float* fit;          // [P]

@@ -3,7 +3,7 @@
 // parallel, one warp per subtree and case block), then the cached nodes
 // bottom up, then the fitness of each root.
 #pragma once
-#include "interp.cuh"
+#include "fused.cuh"
 
 // Work item of entry e: the part of its subtree not covered by large
 // children -- the whole subtree when both children are small, else the
@@ -28,26 +28,39 @@ __global__ void k_build_items(DevPop d, const uint32_t* __restrict__ e_tree) {
     }
 }
 
-// Persistent warps over (item, case block) units.  The next unit's index
-// and descriptor are fetched, and its opcodes staged, while the current
-// one is interpreted (two staging buffers per warp).
+// Shared memory of a k_eval_items CTA: the leaf table (first, so that its
+// addresses fit 16 bits), then per warp a stack window and the instruction
+// list of one chunk.
+template <int K, int V>
+struct ItemsLayout {
+    __host__ __device__ static size_t warp_bytes(int W) { return SmemLayout<K>::stack_bytes(W) + FX_CODE_BYTES; }
+    __host__ __device__ static size_t total(int W, uint32_t ncb) {
+        return FxTable<K, V>::bytes(ncb) + GP_WARPS * warp_bytes(W);
+    }
+};
+
+// Persistent warps over (item, case block) units.  The next unit's index,
+// descriptor and first words are fetched while the current one is evaluated.
+// Bound by instruction issue: with the fused interpreter 13.1 warp
+// instructions a node (23.2 node by node), 80 % of the issue slots busy; 500
+// grafted trees of ~1e6 nodes x 48 cases: items 14.4 -> 6.4 ms.  The words are
+// read straight from the tree, a chunk ahead (no staged copy), so a warp
+// needs its stack window and 1 KB: 40 instead of 24 warps per SM at K = 2.
 template <int K, int V>
 __global__ void __launch_bounds__(GP_WARPS * 32) k_eval_items(DevPop d) {
     if (halted(d)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* kc = reinterpret_cast<float*>(smem_raw);
     const int lane = lane_id(), warp = threadIdx.x >> 5;
-    fill_kc(kc, d.consts);
-    fill_kb(kc + 256);
+    FxTable<K, V>::fill(reinterpret_cast<float*>(smem_raw), d.consts, d.ncb);
     __syncthreads();
-    unsigned char* wbase = smem_raw + SmemLayout<K>::kc_bytes + (size_t)warp * SmemLayout<K>::warp_bytes((int)d.W);
-    Ictx<K> c;
-    c.s = reinterpret_cast<float*>(wbase);
-    c.W = (int)d.W;
-    c.maxd = (int)d.maxdepth;
-    c.kc = kc;
-    c.kb = kc + 256;
-    uint8_t* const stage0 = wbase + SmemLayout<K>::stack_bytes((int)d.W);   // two buffers of STAGE_BYTES
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    const uint32_t wb = sm + FxTable<K, V>::bytes(d.ncb) + warp * (uint32_t)ItemsLayout<K, V>::warp_bytes((int)d.W);
+    FxCtx<K> c;
+    c.stack = wb + lane * K * 4;
+    c.code = wb + (uint32_t)SmemLayout<K>::stack_bytes((int)d.W);
+    c.lo = lane * K * 4;
+    c.W = d.W;
+    c.maxd = d.maxdepth;
     const uint32_t gwarp = blockIdx.x * GP_WARPS + warp;
     c.g = d.ovf + (size_t)gwarp * (d.maxdepth - d.W) * 32 * K;
     const uint32_t ne = d.e_off[d.P];
@@ -55,44 +68,41 @@ __global__ void __launch_bounds__(GP_WARPS * 32) k_eval_items(DevPop d) {
     const uint32_t nunits = ne * d.ncb;
     unsigned long long ops_done = 0;     // nodes interpreted (once per item, not per case block)
 
-    auto grab = [&](uint32_t& u, uint4& desc) {
+    uint32_t un, wa, wl;
+    uint4 dn;
+    auto grab = [&]() {
         uint32_t v = 0;
         if (lane == 0) v = atomicAdd(&d.q[Q_ITEMS], 1u);
-        u = __shfl_sync(FULL, v, 0);
-        desc = make_uint4(0, 0, 0, 0);
-        if (u < nunits) desc = d.it_desc[d.order[u / d.ncb]];
+        un = __shfl_sync(FULL, v, 0);
+        dn = make_uint4(0, 0, 0, 0);
+        if (un < nunits) dn = d.it_desc[d.order[un / d.ncb]];
     };
-    uint32_t un;
-    uint4 dn;
-    grab(un, dn);
-    if (un < nunits && dn.y) stage_issue(stage0, d.arena + (size_t)dn.w * d.cap, dn.x, dn.x + dn.y);
-    cp_async_commit();
-    int cur = 0;
+    auto words = [&]() {
+        if (dn.y) {
+            const uint32_t* tree = reinterpret_cast<const uint32_t*>(d.arena + (size_t)dn.w * d.cap);
+            fx_first([&](uint32_t q) { return __ldg(tree + (q >> 2)); }, dn.x, dn.x + dn.y, wa, wl);
+        }
+    };
+    grab();
+    words();
     while (un < nunits) {
-        const uint32_t u = un;
+        const uint32_t u = un, w0 = wa, w1 = wl;
         const uint4 desc = dn;
-        grab(un, dn);
-        if (un < nunits && dn.y) stage_issue(stage0 + (cur ^ 1) * STAGE_BYTES, d.arena + (size_t)dn.w * d.cap, dn.x, dn.x + dn.y);
-        cp_async_commit();
-        cp_async_wait<1>();
-        __syncwarp();
+        grab();
+        words();
         if (desc.y) {
             const uint32_t cbk = u % d.ncb;
-            load_cases<K>(d, cbk, c.xv);
-            Istate<K> st;
-#pragma unroll
-            for (int k = 0; k < K; ++k) st.acc[k] = 0.f;
-            st.sp = 0;
-            st.ok = true;
-            interp_staged<K, V>(stage0 + cur * STAGE_BYTES, desc.x, desc.x + desc.y, st, c);
-            if (!st.ok && lane == 0) set_status(d.status, ST_STACK);
-            store_slot<K>(d, desc.z, cbk, st.acc);
+            load_cases<K>(d, cbk, c.x);
+            c.lt = FxTable<K, V>::at(sm, cbk);
+            const uint32_t* tree = reinterpret_cast<const uint32_t*>(d.arena + (size_t)desc.w * d.cap);
+            float a[K];
+            const bool ok = fx_run<K, V>([&](uint32_t q) { return __ldg(tree + (q >> 2)); }, desc.x, desc.x + desc.y, w0, w1,
+                                         c, a);
+            if (!ok && lane == 0) set_status(d.status, ST_STACK);
+            store_slot<K>(d, desc.z, cbk, a);
             if (cbk == 0) ops_done += desc.y;
         }
-        __syncwarp();
-        cur ^= 1;
     }
-    cp_async_wait<0>();
     if (lane == 0 && ops_done) { atomicAdd(&d.acc_ops[0], ops_done); atomicAdd(&d.acc_ops[2], ops_done); }
 }
 

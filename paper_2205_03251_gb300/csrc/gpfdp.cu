@@ -274,7 +274,7 @@ auto with_kind(const DevPop& d, F&& f) {
 
 template <int K, int V>
 int setup_items_kernel(gp_pop* pop) {
-    size_t smem = SmemLayout<K>::total((int)pop->d.W, GP_WARPS);
+    size_t smem = ItemsLayout<K, V>::total((int)pop->d.W, pop->d.ncb);
     int max_optin = 0;
     CK(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, pop->dev));
     if (smem > (size_t)max_optin)
@@ -843,7 +843,13 @@ int gp_pop_create(const gp_config* cfg_in, const float* x, const float* targets,
     // (integer set: the caller's int32 bits, copied as they are; Boolean: the
     // target's case words, bit l of word w for case 32w + l)
     std::vector<float> xp(d.Cpad, 0.0f), tp(d.C, 0.0f);
-    if (!boolean) { memcpy(xp.data(), x, sizeof(float) * d.C); memcpy(tp.data(), targets, sizeof(float) * d.C); }
+    if (!boolean) {
+        memcpy(xp.data(), x, sizeof(float) * d.C);
+        // the padded cases repeat the last one: their values are never read, and an input of zero there would send
+        // most divisions of a warp down the slow path of subnormal and special operands
+        for (uint32_t c = d.C; c < d.Cpad; ++c) memcpy(&xp[c], x + d.C - 1, sizeof(float));
+        memcpy(tp.data(), targets, sizeof(float) * d.C);
+    }
     else {
         for (uint32_t w = 0; w < d.C; ++w) {
             uint32_t word = 0;
