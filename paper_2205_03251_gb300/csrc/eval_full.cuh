@@ -41,13 +41,14 @@ struct ItemsLayout {
 
 // Persistent warps over (item, case block) units.  The next unit's index,
 // descriptor and first words are fetched while the current one is evaluated.
-// Bound by instruction issue: with the fused interpreter 13.1 warp
-// instructions a node (23.2 node by node), 80 % of the issue slots busy; 500
-// grafted trees of ~1e6 nodes x 48 cases: items 14.4 -> 6.4 ms.  The words are
-// read straight from the tree, a chunk ahead (no staged copy), so a warp
-// needs its stack window and 1 KB: 40 instead of 24 warps per SM at K = 2.
+// Bound by the indirect branch of each instruction (about 24 cycles of an
+// SM quarter, whatever it branches to; 0.53 instructions a node on grafted
+// trees), which 16 warps per SM saturate.  500 grafted trees of ~1e6 nodes x
+// 48 cases: 14.4 ms node by node, 6.6 ms now; 2,001 uneven integer trees 1.59
+// -> 0.95 ms; 600 uneven trees x 1,000 cases 5.57 -> 3.2 ms.  The words are
+// read straight from the tree, a chunk ahead (no staged copy).
 template <int K, int V>
-__global__ void __launch_bounds__(GP_WARPS * 32) k_eval_items(DevPop d) {
+__global__ void __launch_bounds__(GP_WARPS * 32, K == 4 ? 3 : V == VF ? 4 : 5) k_eval_items(DevPop d) {
     if (halted(d)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
@@ -62,46 +63,59 @@ __global__ void __launch_bounds__(GP_WARPS * 32) k_eval_items(DevPop d) {
     c.W = d.W;
     c.maxd = d.maxdepth;
     const uint32_t gwarp = blockIdx.x * GP_WARPS + warp;
-    c.g = d.ovf + (size_t)gwarp * (d.maxdepth - d.W) * 32 * K;
+    c.g = d.ovf + (size_t)gwarp * d.maxdepth * 32 * K;
     const uint32_t ne = d.e_off[d.P];
     if (ne > d.Ecap) return;
     const uint32_t nunits = ne * d.ncb;
     unsigned long long ops_done = 0;     // nodes interpreted (once per item, not per case block)
 
-    uint32_t un, wa, wl;
-    uint4 dn;
-    auto grab = [&]() {
-        uint32_t v = 0;
-        if (lane == 0) v = atomicAdd(&d.q[Q_ITEMS], 1u);
-        un = __shfl_sync(FULL, v, 0);
-        dn = make_uint4(0, 0, 0, 0);
-        if (un < nunits) dn = d.it_desc[d.order[un / d.ncb]];
+    // Three units are under way in a warp: the one being evaluated, the next
+    // one's first words in flight, and the descriptor of the one after it.
+    // The first unit of each warp is its own (spread over the CTAs, so that a
+    // small population uses every SM), the others come from the queue.
+    const uint32_t nwarps = gridDim.x * GP_WARPS;
+    uint32_t qnext = 0;                                  // lane 0: a unit taken from the queue ahead
+    if (lane == 0) qnext = nwarps + atomicAdd(&d.q[Q_ITEMS], 1u);
+    auto unit = [&]() -> uint32_t {
+        const uint32_t u = __shfl_sync(FULL, qnext, 0);
+        if (lane == 0 && u < nunits) qnext = nwarps + atomicAdd(&d.q[Q_ITEMS], 1u);
+        return u;
     };
-    auto words = [&]() {
-        if (dn.y) {
-            const uint32_t* tree = reinterpret_cast<const uint32_t*>(d.arena + (size_t)dn.w * d.cap);
-            fx_first([&](uint32_t q) { return __ldg(tree + (q >> 2)); }, dn.x, dn.x + dn.y, wa, wl);
+    // a descriptor under way is one register: lane k holds word k
+    auto fetch = [&](uint32_t u) -> uint32_t {
+        return (u < nunits && lane < 4) ? reinterpret_cast<const uint32_t*>(d.it_desc)[4 * (size_t)(u / d.ncb) + lane] : 0u;
+    };
+    auto words = [&](uint32_t t, uint32_t& a0, uint32_t& a1) {
+        const uint32_t s = __shfl_sync(FULL, t, 0), len = __shfl_sync(FULL, t, 1), buf = __shfl_sync(FULL, t, 3);
+        a0 = a1 = 0xFFFFFFFFu;
+        if (len) {
+            const uint32_t* tree = reinterpret_cast<const uint32_t*>(d.arena + (size_t)buf * d.cap);
+            fx_first([&](uint32_t q) { return __ldg(tree + (q >> 2)); }, s, s + len, a0, a1);
         }
     };
-    grab();
-    words();
-    while (un < nunits) {
-        const uint32_t u = un, w0 = wa, w1 = wl;
-        const uint4 desc = dn;
-        grab();
-        words();
-        if (desc.y) {
-            const uint32_t cbk = u % d.ncb;
+    uint32_t u0 = warp * gridDim.x + blockIdx.x, w0, w1;
+    uint32_t t0 = fetch(u0);
+    uint32_t u1 = unit(), t1 = fetch(u1);
+    words(t0, w0, w1);
+    while (u0 < nunits) {
+        uint32_t v0, v1;
+        words(t1, v0, v1);
+        const uint32_t u2 = unit();
+        const uint32_t t2 = fetch(u2);
+        const uint32_t s = __shfl_sync(FULL, t0, 0), len = __shfl_sync(FULL, t0, 1);
+        if (len) {
+            const uint32_t cbk = u0 % d.ncb;
             load_cases<K>(d, cbk, c.x);
             c.lt = FxTable<K, V>::at(sm, cbk);
-            const uint32_t* tree = reinterpret_cast<const uint32_t*>(d.arena + (size_t)desc.w * d.cap);
+            const uint32_t* tree = reinterpret_cast<const uint32_t*>(d.arena + (size_t)__shfl_sync(FULL, t0, 3) * d.cap);
             float a[K];
-            const bool ok = fx_run<K, V>([&](uint32_t q) { return __ldg(tree + (q >> 2)); }, desc.x, desc.x + desc.y, w0, w1,
-                                         c, a);
+            const bool ok = fx_run<K, V>([&](uint32_t q) { return __ldg(tree + (q >> 2)); }, s, s + len, w0, w1, c, a);
             if (!ok && lane == 0) set_status(d.status, ST_STACK);
-            store_slot<K>(d, desc.z, cbk, a);
-            if (cbk == 0) ops_done += desc.y;
+            store_slot<K>(d, __shfl_sync(FULL, t0, 2), cbk, a);
+            if (cbk == 0) ops_done += len;
         }
+        u0 = u1; t0 = t1; w0 = v0; w1 = v1;
+        u1 = u2; t1 = t2;
     }
     if (lane == 0 && ops_done) { atomicAdd(&d.acc_ops[0], ops_done); atomicAdd(&d.acc_ops[2], ops_done); }
 }

@@ -16,13 +16,14 @@
 // their own.  Every opcode is still applied to every test case, to the same
 // operands in the same order: the values are the same bits.
 //
-// Stack depth: B(q), the number of complete subtrees in [q, end), is the
+// Stack depth: B(q), the number of complete subtrees in [q, end), bounds the
 // number of entries between two instructions (one of them the initial
-// running value).  The decoder knows it, so the executor has no checks: a
-// chunk of 128 nodes whose depths stay within the shared window runs on it
-// alone, any other chunk on a checked path with the global overflow area,
-// and a malformed run (B negative somewhere, or not 1 at its start) is
-// refused before anything is executed that could leave the stack.
+// running value).  The decoder knows it, so the executor has no checks: the
+// window of W entries in shared memory slides over the stack from chunk to
+// chunk (entries below it in a global overflow area), and a chunk of 128
+// nodes whose depths span more than the window runs on the global area alone.
+// A malformed run (B negative somewhere, or not 1 at its start) is refused
+// before anything is executed that could leave the stack.
 #pragma once
 #include "interp.cuh"
 
@@ -54,6 +55,11 @@ __device__ __forceinline__ uint32_t fx_zero_bytes(uint32_t t) {
 __device__ __forceinline__ uint32_t fx_funcs(uint32_t w) { return fx_zero_bytes(w & 0xFCFCFCFCu); }
 
 __device__ __forceinline__ void fx_sts(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v)); }
+// instruction `idx` at the list address `at` and its operand one word on, if `on` is not zero (predicated: no branch)
+__device__ __forceinline__ void fx_put(uint32_t on, uint32_t at, uint32_t idx, uint32_t y) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u32 [%1], %2;\n\t@p st.shared.u32 [%1+12], %3;\n\t}"
+                 ::"r"(on), "r"(at), "r"(idx), "r"(y));
+}
 
 // The lane's word of a chunk: bytes [q, q + 4) of the run [s, e), positions
 // outside the run replaced by 0xFF (a leaf).  `ld(q)` reads the word at q, a
@@ -76,19 +82,19 @@ struct FxCarry {
 
 struct FxChunk {
     uint32_t n;          // instructions, including the captures' end marks
-    bool over, bad;      // deeper than the window; malformed
+    int32_t in, mx, mn;  // B before the chunk (uniform); largest and smallest B after this lane's nodes
+    bool bad;            // malformed
 };
 
 // Decode the chunk at `base` (c.w, c.f; fl: the mask of the chunk to the
 // left) into the list at shared address `code`.  word j holds the index of
 // instruction j and the operand of instruction j - 1, so that the executor
 // has the index of the next instruction one instruction early.  lt: shared
-// address of the leaf table (constants: 4 bytes per opcode; Boolean: LS bytes
-// per input).  caps: 0x01 in the bytes of nodes after which the list is
+// address of the leaf table, LS bytes per opcode.  caps: 0x01 in the bytes of nodes after which the list is
 // interrupted by an end mark (CAP).
 template <int V, bool CAP, int LS>
 __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32_t base, uint32_t s, uint32_t e,
-                                             uint32_t W, uint32_t code, uint32_t lt, uint32_t caps) {
+                                             uint32_t code, uint32_t lt, uint32_t caps) {
     const int lane = lane_id();
     const int32_t q = base + 4 * lane;
     const uint32_t w = c.w, f = c.f;
@@ -129,15 +135,16 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     const uint32_t all = __shfl_sync(FULL, sum, 0);
     const uint32_t right = sum - own;
     const int b0 = c.B + ((int32_t)right >> 16);
-    const int mx = b0 + max(max(d3, d2), max(d1, d0)), mn = b0 + min(min(d3, d2), min(d1, d0));
     FxChunk r;
     r.n = all & 0xFFFFu;
-    r.over = c.B > (int)W || __any_sync(FULL, mx > (int)W);      // before the chunk's first node, or after any of them
+    r.in = c.B;
+    r.mx = b0 + max(max(d3, d2), max(d1, d0));
+    r.mn = b0 + min(min(d3, d2), min(d1, d0));
     c.B += (int32_t)all >> 16;
     // a function among the last two nodes of the run has no operands
     const int32_t last2 = (int32_t)e - 2 - q;
     const bool tail = (valid & f) != 0 && last2 < 4 && (valid & f & (last2 <= 0 ? 0xFFFFFFFFu : 0xFFFFFFFFu << (8 * last2))) != 0;
-    r.bad = __any_sync(FULL, mn < 0 || tail);
+    r.bad = __any_sync(FULL, r.mn < 0 || tail);
     // instruction indexes of the four bytes at once
     uint32_t idx, A;                     // index; the byte of the first operand
     uint32_t both = 0;                   // f L L with two table operands
@@ -163,19 +170,18 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     }
     // the lane's instructions in execution order: from its last byte down
     uint32_t at = code + ((right & 0xFFFFu) << 3);
-    const uint32_t size = (V == VB) ? (uint32_t)LS : 4u, most = (V == VB) ? FX_BROWS - 1u : 0xFFu;
+    const uint32_t size = (uint32_t)LS, most = (V == VB) ? FX_BROWS - 1u : 0xFFu;
 #pragma unroll
     for (int j = 3; j >= 0; --j) {
-        if (head & (1u << (8 * j))) {
-            uint32_t y = lt + ((A >> (8 * j)) & most) * size;
-            if (both & (1u << (8 * j))) y |= (lt + ((n2 >> (8 * j)) & most) * size) << 16;
-            fx_sts(at, (idx >> (8 * j)) & 0xFFu);
-            fx_sts(at + 12, y);
-            at += 8;
-            if (CAP && (caps & (1u << (8 * j)))) {
-                fx_sts(at, FX_EXIT);
-                at += 8;
-            }
+        const uint32_t on = head & (1u << (8 * j));
+        const uint32_t second = (lt << 16) + ((n2 >> (8 * j)) & most) * (size << 16);
+        const uint32_t y = lt + ((A >> (8 * j)) & most) * size + ((both & (1u << (8 * j))) ? second : 0u);
+        fx_put(on, at, (idx >> (8 * j)) & 0xFFu, y);
+        at += on ? 8u : 0u;
+        if (CAP) {
+            const uint32_t cap = caps & (1u << (8 * j));
+            if (cap) fx_sts(at, FX_EXIT);
+            at += cap ? 8u : 0u;
         }
     }
     if (lane == 0) fx_sts(code + (r.n << 3), FX_EXIT);
@@ -186,92 +192,139 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
 // ---- executor
 //
 // One block of PTX: every instruction ends with an indirect branch to the
-// next (declared uniform: all lanes read the same list).  Registers: a0.. the
-// running value, x0.. the inputs, sa the next free stack entry, ip the list;
+// next (declared uniform: all lanes read the same list).  Registers: a.. the
+// running value, x.. the inputs, sa the next free stack entry, ip the list;
 // nx is the index of the next instruction, loaded one instruction early.
-#define FX1(ins, d, a, b) ins " " d "0, " a "0, " b "0;\n\t"
-#define FX2(ins, d, a, b) FX1(ins, d, a, b) ins " " d "1, " a "1, " b "1;\n\t"
-#define FX4(ins, d, a, b) FX2(ins, d, a, b) ins " " d "2, " a "2, " b "2;\n\t" ins " " d "3, " a "3, " b "3;\n\t"
-// second or first operand the same register for all cases
-#define FXR1(ins, d, a, b) ins " " d "0, " a "0, " b ";\n\t"
-#define FXR2(ins, d, a, b) FXR1(ins, d, a, b) ins " " d "1, " a "1, " b ";\n\t"
-#define FXR4(ins, d, a, b) FXR2(ins, d, a, b) ins " " d "2, " a "2, " b ";\n\t" ins " " d "3, " a "3, " b ";\n\t"
-#define FXL1(ins, d, a, b) ins " " d "0, " a ", " b "0;\n\t"
-#define FXL2(ins, d, a, b) FXL1(ins, d, a, b) ins " " d "1, " a ", " b "1;\n\t"
-#define FXL4(ins, d, a, b) FXL2(ins, d, a, b) ins " " d "2, " a ", " b "2;\n\t" ins " " d "3, " a ", " b "3;\n\t"
-#define FXM1(d, a) "mov.b32 " d "0, " a "0;\n\t"
-#define FXM2(d, a) FXM1(d, a) "mov.b32 " d "1, " a "1;\n\t"
-#define FXM4(d, a) FXM2(d, a) "mov.b32 " d "2, " a "2;\n\tmov.b32 " d "3, " a "3;\n\t"
-#define FXB1(d, a) "mov.b32 " d "0, " a ";\n\t"
-#define FXB2(d, a) FXB1(d, a) "mov.b32 " d "1, " a ";\n\t"
-#define FXB4(d, a) FXB2(d, a) "mov.b32 " d "2, " a ";\n\tmov.b32 " d "3, " a ";\n\t"
-#define FXV1(r) "{" r "0}"
-#define FXV2(r) "{" r "0, " r "1}"
-#define FXV4(r) "{" r "0, " r "1, " r "2, " r "3}"
-#define FXLD1 "ld.shared.b32 "
-#define FXLD2 "ld.shared.v2.b32 "
-#define FXLD4 "ld.shared.v4.b32 "
-#define FXST1 "st.shared.b32 "
-#define FXST2 "st.shared.v2.b32 "
-#define FXST4 "st.shared.v4.b32 "
-#define FXSV1(r) r "0"
-#define FXSV2(r) FXV2(r)
-#define FXSV4(r) FXV4(r)
-#define FXBY1 "128"
-#define FXBY2 "256"
-#define FXBY4 "512"
+//
+// A value of K cases is K 32-bit registers (form S1, S2), or for the
+// binary32 set at K = 2 and 4 one or two pairs (P2, P4) on which one
+// instruction computes two cases; there the table holds each constant twice.
+//
+// Operations over a whole value (d, a, b: register prefixes; c: one register
+// or pair for all cases):
+//   FXO_f(ins, d, a, b)   FXR_f(ins, d, a, c)   FXL_f(ins, d, c, b)   FXM_f(d, a)   FXB_f(d, c)
+#define FXO_S1(ins, d, a, b) ins " " d "0, " a "0, " b "0;\n\t"
+#define FXR_S1(ins, d, a, c) ins " " d "0, " a "0, " c ";\n\t"
+#define FXL_S1(ins, d, c, b) ins " " d "0, " c ", " b "0;\n\t"
+#define FXM_S1(d, a) "mov.b32 " d "0, " a "0;\n\t"
+#define FXB_S1(d, c) "mov.b32 " d "0, " c ";\n\t"
+#define FXO_S2(ins, d, a, b) FXO_S1(ins, d, a, b) ins " " d "1, " a "1, " b "1;\n\t"
+#define FXR_S2(ins, d, a, c) FXR_S1(ins, d, a, c) ins " " d "1, " a "1, " c ";\n\t"
+#define FXL_S2(ins, d, c, b) FXL_S1(ins, d, c, b) ins " " d "1, " c ", " b "1;\n\t"
+#define FXM_S2(d, a) FXM_S1(d, a) "mov.b32 " d "1, " a "1;\n\t"
+#define FXB_S2(d, c) FXB_S1(d, c) "mov.b32 " d "1, " c ";\n\t"
+#define FXO_P2(ins, d, a, b) FXO_S1(ins, d, a, b)
+#define FXR_P2(ins, d, a, c) FXR_S1(ins, d, a, c)
+#define FXL_P2(ins, d, c, b) FXL_S1(ins, d, c, b)
+#define FXM_P2(d, a) "mov.b64 " d "0, " a "0;\n\t"
+#define FXB_P2(d, c) "mov.b64 " d "0, " c ";\n\t"
+#define FXO_P4(ins, d, a, b) FXO_S2(ins, d, a, b)
+#define FXR_P4(ins, d, a, c) FXR_S2(ins, d, a, c)
+#define FXL_P4(ins, d, c, b) FXL_S2(ins, d, c, b)
+#define FXM_P4(d, a) FXM_P2(d, a) "mov.b64 " d "1, " a "1;\n\t"
+#define FXB_P4(d, c) FXB_P2(d, c) "mov.b64 " d "1, " c ";\n\t"
+// one value from or to shared memory, and its stride on the stack
+#define FXLD_S1(r, at) "ld.shared.b32 " r "0, [" at "];\n\t"
+#define FXST_S1(at, r) "st.shared.b32 [" at "], " r "0;\n\t"
+#define FXLD_S2(r, at) "ld.shared.v2.b32 {" r "0, " r "1}, [" at "];\n\t"
+#define FXST_S2(at, r) "st.shared.v2.b32 [" at "], {" r "0, " r "1};\n\t"
+#define FXLD_P2(r, at) "ld.shared.b64 " r "0, [" at "];\n\t"
+#define FXST_P2(at, r) "st.shared.b64 [" at "], " r "0;\n\t"
+#define FXLD_P4(r, at) "ld.shared.v2.b64 {" r "0, " r "1}, [" at "];\n\t"
+#define FXST_P4(at, r) "st.shared.v2.b64 [" at "], {" r "0, " r "1};\n\t"
+#define FXBY_S1 "128"
+#define FXBY_S2 "256"
+#define FXBY_P2 "256"
+#define FXBY_P4 "512"
+// one constant
+#define FXC_S1(r, at) "ld.shared.b32 " r ", [" at "];\n\t"
+#define FXC_S2(r, at) FXC_S1(r, at)
+#define FXC_P2(r, at) "ld.shared.b64 " r ", [" at "];\n\t"
+#define FXC_P4(r, at) FXC_P2(r, at)
 
 #define FX_NEXT "mov.b32 nx, ix;\n\tld.shared.v2.b32 {ix, oy}, [ip];\n\tadd.u32 ip, ip, 8;\n\t"
 #define FX_GO "brx.idx.uni nx, FXT;\n"
-#define FX_PUSH(K) FXST##K "[sa], " FXSV##K("a") ";\n\tadd.u32 sa, sa, " FXBY##K ";\n\t"
-#define FX_POP(K) "sub.u32 sa, sa, " FXBY##K ";\n\t" FXLD##K FXSV##K("r") ", [sa];\n\t"
-#define FX_CST "ld.shared.b32 c0, [oy];\n\t"
-#define FX_TWO "and.b32 t, oy, 0xFFFF;\n\tshr.u32 u, oy, 16;\n\tld.shared.b32 c0, [t];\n\tld.shared.b32 c1, [u];\n\t"
+#define FX_PUSH(F) FXST_##F("sa", "a") "add.u32 sa, sa, " FXBY_##F ";\n\t"
+#define FX_POP(F) "sub.u32 sa, sa, " FXBY_##F ";\n\t" FXLD_##F("r", "sa")
+#define FX_CST(F) FXC_##F("c0", "oy")
+#define FX_TWO(F) "and.b32 t, oy, 0xFFFF;\n\tshr.u32 u, oy, 16;\n\t" FXC_##F("c0", "t") FXC_##F("c1", "u")
 
-// the twelve instructions of a function that is one machine instruction `ins`: labels L<b>.. for f L L, M<b>.. for
-// f L ., P<b> for f f ..
-#define FX_FUNC(K, o, ins)                                                                                          \
-    "FXA" o "0:\n\t" FX_NEXT FX_PUSH(K) FX##K(ins, "a", "x", "x") FX_GO                                              \
-    "FXA" o "1:\n\t" FX_CST FX_NEXT FX_PUSH(K) FXR##K(ins, "a", "x", "c0") FX_GO                                     \
-    "FXA" o "2:\n\t" FX_CST FX_NEXT FX_PUSH(K) FXL##K(ins, "a", "c0", "x") FX_GO                                     \
-    "FXA" o "3:\n\t" FX_TWO FX_NEXT FX_PUSH(K) ins " c0, c0, c1;\n\t" FXB##K("a", "c0") FX_GO                        \
-    "FXM" o "0:\n\t" FX_NEXT FX##K(ins, "a", "x", "a") FX_GO                                                         \
-    "FXM" o "1:\n\t" FX_CST FX_NEXT FXL##K(ins, "a", "c0", "a") FX_GO                                                \
-    "FXP" o "0:\n\t" FX_NEXT FX_POP(K) FX##K(ins, "a", "a", "r") FX_GO
-// a function of several machine instructions: operands to n.. and r.., then the shared body at FXDV
-#define FX_LONG(K, o)                                                                                               \
-    "FXA" o "0:\n\t" FX_NEXT FX_PUSH(K) FXM##K("n", "x") FXM##K("r", "x") "bra.uni FXDV;\n"                          \
-    "FXA" o "1:\n\t" FX_CST FX_NEXT FX_PUSH(K) FXM##K("n", "x") FXB##K("r", "c0") "bra.uni FXDV;\n"                  \
-    "FXA" o "2:\n\t" FX_CST FX_NEXT FX_PUSH(K) FXB##K("n", "c0") FXM##K("r", "x") "bra.uni FXDV;\n"                  \
-    "FXA" o "3:\n\t" FX_TWO FX_NEXT FX_PUSH(K) FXB##K("n", "c0") FXB##K("r", "c1") "bra.uni FXDV;\n"                 \
-    "FXM" o "0:\n\t" FX_NEXT FXM##K("r", "a") FXM##K("n", "x") "bra.uni FXDV;\n"                                     \
-    "FXM" o "1:\n\t" FX_CST FX_NEXT FXM##K("r", "a") FXB##K("n", "c0") "bra.uni FXDV;\n"                             \
-    "FXP" o "0:\n\t" FX_NEXT FX_POP(K) FXM##K("n", "a") "bra.uni FXDV;\n"
-// protected division: 1 for a zero divisor, without dividing by it (1 / 1)
-#define FX_FDIV1(k) "setp.eq.f32 p, r" #k ", 0f00000000;\n\tselp.b32 n" #k ", 0x3F800000, n" #k ", p;\n\t"          \
-                    "selp.b32 r" #k ", 0x3F800000, r" #k ", p;\n\tdiv.rn.f32 a" #k ", n" #k ", r" #k ";\n\t"
-#define FX_FDIVS1 FX_FDIV1(0)
-#define FX_FDIVS2 FX_FDIV1(0) FX_FDIV1(1)
-#define FX_FDIVS4 FX_FDIV1(0) FX_FDIV1(1) FX_FDIV1(2) FX_FDIV1(3)
+// The seven instructions of a function that is one machine instruction (o:
+// its number): labels FXA for f L L by leaf kinds, FXM for f L ., FXP for f f ..
+#define FX_FUNC(F, o, ins)                                                                                          \
+    "FXA" o "0:\n\t" FX_NEXT FX_PUSH(F) FXO_##F(ins, "a", "x", "x") FX_GO                                            \
+    "FXA" o "1:\n\t" FX_CST(F) FX_NEXT FX_PUSH(F) FXR_##F(ins, "a", "x", "c0") FX_GO                                 \
+    "FXA" o "2:\n\t" FX_CST(F) FX_NEXT FX_PUSH(F) FXL_##F(ins, "a", "c0", "x") FX_GO                                 \
+    "FXA" o "3:\n\t" FX_TWO(F) FX_NEXT FX_PUSH(F) ins " c0, c0, c1;\n\t" FXB_##F("a", "c0") FX_GO                    \
+    "FXM" o "0:\n\t" FX_NEXT FXO_##F(ins, "a", "x", "a") FX_GO                                                       \
+    "FXM" o "1:\n\t" FX_CST(F) FX_NEXT FXL_##F(ins, "a", "c0", "a") FX_GO                                            \
+    "FXP" o "0:\n\t" FX_NEXT FX_POP(F) FXO_##F(ins, "a", "a", "r") FX_GO
+// Division: operands to n.. and r.., then the shared body at FXDV.
+#define FX_LONG(F, o)                                                                                               \
+    "FXA" o "0:\n\t" FX_NEXT FX_PUSH(F) FXM_##F("n", "x") FXM_##F("r", "x") "bra.uni FXDV;\n"                        \
+    "FXA" o "1:\n\t" FX_CST(F) FX_NEXT FX_PUSH(F) FXM_##F("n", "x") FXB_##F("r", "c0") "bra.uni FXDV;\n"             \
+    "FXA" o "2:\n\t" FX_CST(F) FX_NEXT FX_PUSH(F) FXB_##F("n", "c0") FXM_##F("r", "x") "bra.uni FXDV;\n"             \
+    "FXA" o "3:\n\t" FX_TWO(F) FX_NEXT FX_PUSH(F) FXB_##F("n", "c0") FXB_##F("r", "c1") "bra.uni FXDV;\n"            \
+    "FXM" o "0:\n\t" FX_NEXT FXM_##F("r", "a") FXM_##F("n", "x") "bra.uni FXDV;\n"                                   \
+    "FXM" o "1:\n\t" FX_CST(F) FX_NEXT FXM_##F("r", "a") FXB_##F("n", "c0") "bra.uni FXDV;\n"                        \
+    "FXP" o "0:\n\t" FX_NEXT FX_POP(F) FXM_##F("n", "a") "bra.uni FXDV;\n"
+
+// Protected binary32 division.  When every operand of the warp lies within
+// [2^-60, 2^60] no step below can overflow or lose bits, and the quotient is
+// Markstein's (IBM J. Res. Dev. 34, 1990): y an approximate reciprocal, one
+// Newton step y += y (1 - b y), q = a y, q += y (a - b q).  For this
+// machine's rcp.approx it is the correctly rounded quotient for all 2^46
+// pairs of significands (every pair was compared with its remainder); the
+// scale of the operands does not change a bit of it.  Without the Newton step
+// 79,381 pairs would be one unit off.  Any other operand -- zero, tiny, huge,
+// not finite -- sends the warp to FXDR: 1 for a zero divisor (as 1 / 1), else
+// the machine's division.
+#define FXD_IN(v, w, z) "max.NaN.f32 h, " v ", " w ", " z ";\n\tmin.f32 l, " v ", " w ", " z ";\n\t"
+#define FXD_MORE2(v, w) "max.NaN.f32 h, h, " v ", " w ";\n\tmin.f32 l, l, " v ", " w ";\n\t"
+#define FXD_ONE(k) "setp.eq.f32 p, d" #k ", 0f00000000;\n\tselp.b32 m" #k ", 0x3F800000, m" #k ", p;\n\t"           \
+                   "selp.b32 d" #k ", 0x3F800000, d" #k ", p;\n\tdiv.rn.f32 m" #k ", m" #k ", d" #k ";\n\t"
+#define FXD_TEST "setp.le.f32 p, h, 0f5D800000;\n\tsetp.ge.and.f32 p, l, 0f21800000, p;\n\t"                        \
+                 "vote.sync.all.pred p, p, 0xFFFFFFFF;\n\t@!p bra.uni FXDR;\n\t"
+#define FXD_ABS(k) "abs.f32 e" #k ", m" #k ";\n\tabs.f32 g" #k ", d" #k ";\n\t"
+#define FXD_PAIR(i, ka, kb) /* pair i holds cases ka and kb; m: numerators, d: divisors */                          \
+    "rcp.approx.ftz.f32 e" #ka ", d" #ka ";\n\trcp.approx.ftz.f32 e" #kb ", d" #kb ";\n\tmov.b64 y, {e" #ka ", e" #kb "};\n\t" \
+    "xor.b64 v, r" #i ", 0x8000000080000000;\n\tfma.rn.f32x2 z, v, y, one;\n\tfma.rn.f32x2 y, y, z, y;\n\t"          \
+    "mul.rn.f32x2 q, n" #i ", y;\n\tfma.rn.f32x2 z, v, q, n" #i ";\n\tfma.rn.f32x2 a" #i ", z, y, q;\n\t"
+#define FXDIV_S1                                                                                                    \
+    "mov.b32 m0, n0;\n\tmov.b32 d0, r0;\n\t" FXD_ABS(0)                                                              \
+    "max.NaN.f32 h, e0, g0;\n\tmin.f32 l, e0, g0;\n\t" FXD_TEST                                                      \
+    "rcp.approx.ftz.f32 e0, d0;\n\tneg.f32 g0, d0;\n\tfma.rn.f32 h, g0, e0, 0f3F800000;\n\tfma.rn.f32 e0, e0, h, e0;\n\t" \
+    "mul.rn.f32 h, m0, e0;\n\tfma.rn.f32 l, g0, h, m0;\n\tfma.rn.f32 a0, l, e0, h;\n\t" FX_GO                        \
+    "FXDR:\n\t" FXD_ONE(0) "mov.b32 a0, m0;\n\t" FX_GO
+#define FXDIV_P2                                                                                                    \
+    "mov.b64 {m0, m1}, n0;\n\tmov.b64 {d0, d1}, r0;\n\t" FXD_ABS(0) FXD_ABS(1)                                       \
+    FXD_IN("e0", "e1", "g0") "max.NaN.f32 h, h, g1;\n\tmin.f32 l, l, g1;\n\t" FXD_TEST FXD_PAIR(0, 0, 1) FX_GO       \
+    "FXDR:\n\t" FXD_ONE(0) FXD_ONE(1) "mov.b64 a0, {m0, m1};\n\t" FX_GO
+#define FXDIV_P4                                                                                                    \
+    "mov.b64 {m0, m1}, n0;\n\tmov.b64 {d0, d1}, r0;\n\tmov.b64 {m2, m3}, n1;\n\tmov.b64 {d2, d3}, r1;\n\t"           \
+    FXD_ABS(0) FXD_ABS(1) FXD_ABS(2) FXD_ABS(3) FXD_IN("e0", "e1", "g0") FXD_MORE2("g1", "e2") FXD_MORE2("e3", "g2") \
+    "max.NaN.f32 h, h, g3;\n\tmin.f32 l, l, g3;\n\t" FXD_TEST FXD_PAIR(0, 0, 1) FXD_PAIR(1, 2, 3) FX_GO              \
+    "FXDR:\n\t" FXD_ONE(0) FXD_ONE(1) FXD_ONE(2) FXD_ONE(3) "mov.b64 a0, {m0, m1};\n\tmov.b64 a1, {m2, m3};\n\t" FX_GO
 // integers: 1 for a zero divisor (1 / 1); INT32_MIN / -1 = INT32_MIN (divided by 1 instead)
 #define FX_IDIV1(k) "setp.eq.s32 p, r" #k ", 0;\n\tselp.b32 n" #k ", 1, n" #k ", p;\n\tselp.b32 r" #k ", 1, r" #k ", p;\n\t" \
                     "setp.eq.s32 p, r" #k ", -1;\n\tsetp.eq.and.s32 p, n" #k ", 0x80000000, p;\n\t"                    \
                     "selp.b32 r" #k ", 1, r" #k ", p;\n\tdiv.s32 a" #k ", n" #k ", r" #k ";\n\t"
-#define FX_IDIVS1 FX_IDIV1(0)
-#define FX_IDIVS2 FX_IDIV1(0) FX_IDIV1(1)
-// Boolean leaves: this lane's words of an input, at the lane's place of the table row
-#define FX_BLD(K, r, a) FXLD##K FXSV##K(r) ", [" a "];\n\t"
-#define FX_BFUNC(K, o, ins, post)                                                                                   \
+#define FX_IDIV_S1 FX_IDIV1(0) FX_GO
+#define FX_IDIV_S2 FX_IDIV1(0) FX_IDIV1(1) FX_GO
+// Boolean: every leaf is a row of the table, at the lane's place
+#define FX_BFUNC(F, o, ins, post)                                                                                   \
     "FXA" o "3:\n\tand.b32 t, oy, 0xFFFF;\n\tshr.u32 u, oy, 16;\n\tadd.u32 t, t, lo;\n\tadd.u32 u, u, lo;\n\t"       \
-    FX_BLD(K, "n", "t") FX_BLD(K, "r", "u") FX_NEXT FX_PUSH(K) FX##K(ins, "a", "n", "r") post FX_GO                  \
-    "FXM" o "1:\n\tadd.u32 t, oy, lo;\n\t" FX_BLD(K, "n", "t") FX_NEXT FX##K(ins, "a", "n", "a") post FX_GO          \
-    "FXP" o "0:\n\t" FX_NEXT FX_POP(K) FX##K(ins, "a", "a", "r") post FX_GO
-#define FXN1 "not.b32 a0, a0;\n\t"
-#define FXN2 FXN1 "not.b32 a1, a1;\n\t"
+    FXLD_##F("n", "t") FXLD_##F("r", "u") FX_NEXT FX_PUSH(F) FXO_##F(ins, "a", "n", "r") post FX_GO                  \
+    "FXM" o "1:\n\tadd.u32 t, oy, lo;\n\t" FXLD_##F("n", "t") FX_NEXT FXO_##F(ins, "a", "n", "a") post FX_GO         \
+    "FXP" o "0:\n\t" FX_NEXT FX_POP(F) FXO_##F(ins, "a", "a", "r") post FX_GO
+#define FXN_S1 "not.b32 a0, a0;\n\t"
+#define FXN_S2 FXN_S1 "not.b32 a1, a1;\n\t"
 
+#define FX_REGS_S ".reg .b32 a0, a1, x0, x1, r0, r1, n0, n1, c0, c1;\n\t"
+#define FX_REGS_P ".reg .b64 a0, a1, x0, x1, r0, r1, n0, n1, c0, c1, y, z, v, q, one;\n\tmov.b64 one, 0x3F8000003F800000;\n\t"
 #define FX_REGS                                                                                                     \
-    ".reg .pred p;\n\t.reg .b32 a0, a1, a2, a3, x0, x1, x2, x3, r0, r1, r2, r3, n0, n1, n2, n3;\n\t"                 \
-    ".reg .b32 c0, c1, ix, oy, nx, t, u, ip, sa, lo;\n\t"
+    ".reg .pred p;\n\t.reg .b32 ix, oy, nx, t, u, ip, sa, lo, h, l, m0, m1, m2, m3, d0, d1, d2, d3;\n\t"             \
+    ".reg .b32 e0, e1, e2, e3, g0, g1, g2, g3;\n\t"
 #define FX_TABLE                                                                                                    \
     "FXT: .branchtargets FXA00, FXA01, FXA02, FXA03, FXA10, FXA11, FXA12, FXA13, FXA20, FXA21, FXA22, FXA23, "       \
     "FXA30, FXA31, FXA32, FXA33, FXM00, FXM01, FXM10, FXM11, FXM20, FXM21, FXM30, FXM31, FXP00, FXP10, FXP20, "      \
@@ -281,53 +334,57 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     "FXA33, FXA33, FXA33, FXA33, FXM01, FXM01, FXM11, FXM11, FXM21, FXM21, FXM31, FXM31, FXP00, FXP10, FXP20, "      \
     "FXP30, FXL1, FXL1, FXEND;\n\t"
 #define FX_START "ld.shared.v2.b32 {ix, oy}, [ip];\n\tadd.u32 ip, ip, 8;\n\t" FX_NEXT FX_GO
-#define FX_LEAVES(K)                                                                                                \
-    "FXL0:\n\t" FX_NEXT FX_PUSH(K) FXM##K("a", "x") FX_GO                                                            \
-    "FXL1:\n\t" FX_CST FX_NEXT FX_PUSH(K) FXB##K("a", "c0") FX_GO
-#define FX_BODY_F(K)                                                                                                \
-    FX_FUNC(K, "0", "add.rn.f32") FX_FUNC(K, "1", "sub.rn.f32") FX_FUNC(K, "2", "mul.rn.f32") FX_LONG(K, "3")        \
-    "FXDV:\n\t" FX_FDIVS##K FX_GO FX_LEAVES(K) "FXEND:\n\tsub.u32 ip, ip, 8;\n\t"
-#define FX_BODY_I(K)                                                                                                \
-    FX_FUNC(K, "0", "add.u32") FX_FUNC(K, "1", "sub.u32") FX_FUNC(K, "2", "mul.lo.u32") FX_LONG(K, "3")              \
-    "FXDV:\n\t" FX_IDIVS##K FX_GO FX_LEAVES(K) "FXEND:\n\tsub.u32 ip, ip, 8;\n\t"
-#define FX_BODY_B(K)                                                                                                \
-    FX_BFUNC(K, "0", "and.b32", "") FX_BFUNC(K, "1", "or.b32", "") FX_BFUNC(K, "2", "and.b32", FXN##K)               \
-    FX_BFUNC(K, "3", "or.b32", FXN##K)                                                                               \
-    "FXL1:\n\tadd.u32 t, oy, lo;\n\t" FX_NEXT FX_PUSH(K) FX_BLD(K, "a", "t") FX_GO                                   \
-    "FXEND:\n\tsub.u32 ip, ip, 8;\n\t"
+#define FX_STOP "FXEND:\n\tsub.u32 ip, ip, 8;\n\t"
+#define FX_LEAVES(F)                                                                                                \
+    "FXL0:\n\t" FX_NEXT FX_PUSH(F) FXM_##F("a", "x") FX_GO                                                           \
+    "FXL1:\n\t" FX_CST(F) FX_NEXT FX_PUSH(F) FXB_##F("a", "c0") FX_GO
+#define FX_BODY_F(F, w)                                                                                             \
+    FX_FUNC(F, "0", "add.rn.f32" w) FX_FUNC(F, "1", "sub.rn.f32" w) FX_FUNC(F, "2", "mul.rn.f32" w) FX_LONG(F, "3")  \
+    "FXDV:\n\t" FXDIV_##F FX_LEAVES(F) FX_STOP
+#define FX_BODY_I(F)                                                                                                \
+    FX_FUNC(F, "0", "add.u32") FX_FUNC(F, "1", "sub.u32") FX_FUNC(F, "2", "mul.lo.u32") FX_LONG(F, "3")              \
+    "FXDV:\n\t" FX_IDIV_##F FX_LEAVES(F) FX_STOP
+#define FX_BODY_B(F)                                                                                                \
+    FX_BFUNC(F, "0", "and.b32", "") FX_BFUNC(F, "1", "or.b32", "") FX_BFUNC(F, "2", "and.b32", FXN_##F)              \
+    FX_BFUNC(F, "3", "or.b32", FXN_##F)                                                                              \
+    "FXL1:\n\tadd.u32 t, oy, lo;\n\t" FX_NEXT FX_PUSH(F) FXLD_##F("a", "t") FX_GO FX_STOP
 
 // Run the list at shared address `ip` up to an end mark; afterwards ip is
 // where to go on from.  lo: the lane's offset in a row of the Boolean table.
 template <int K, int V>
 __device__ __forceinline__ void fx_exec(uint32_t& ip, float (&a)[K], uint32_t& sa, const float (&x)[K], uint32_t lo) {
     if constexpr (K == 1) {
-#define FX_ASM1(TAB, BODY)                                                                                          \
-    asm volatile("{\n\t" FX_REGS TAB "mov.b32 a0, %0;\n\tmov.b32 sa, %1;\n\tmov.b32 ip, %2;\n\t"                     \
+#define FX_ASM(TAB, BODY)                                                                                           \
+    asm volatile("{\n\t" FX_REGS FX_REGS_S TAB "mov.b32 a0, %0;\n\tmov.b32 sa, %1;\n\tmov.b32 ip, %2;\n\t"           \
                  "mov.b32 x0, %3;\n\tmov.b32 lo, %4;\n\t" FX_START BODY                                             \
                  "mov.b32 %0, a0;\n\tmov.b32 %1, sa;\n\tmov.b32 %2, ip;\n\t}"                                        \
                  : "+f"(a[0]), "+r"(sa), "+r"(ip) : "f"(x[0]), "r"(lo) : "memory")
-        if constexpr (V == VF) FX_ASM1(FX_TABLE, FX_BODY_F(1));
-        else if constexpr (V == VI) FX_ASM1(FX_TABLE, FX_BODY_I(1));
-        else FX_ASM1(FX_BTABLE, FX_BODY_B(1));
-    } else if constexpr (K == 2) {
-#define FX_ASM2(TAB, BODY)                                                                                          \
-    asm volatile("{\n\t" FX_REGS TAB "mov.b32 a0, %0;\n\tmov.b32 a1, %1;\n\tmov.b32 sa, %2;\n\tmov.b32 ip, %3;\n\t"  \
-                 "mov.b32 x0, %4;\n\tmov.b32 x1, %5;\n\tmov.b32 lo, %6;\n\t" FX_START BODY                          \
+        if constexpr (V == VF) FX_ASM(FX_TABLE, FX_BODY_F(S1, ""));
+        else if constexpr (V == VI) FX_ASM(FX_TABLE, FX_BODY_I(S1));
+        else FX_ASM(FX_BTABLE, FX_BODY_B(S1));
+#undef FX_ASM
+    } else if constexpr (K == 2 && V != VF) {
+#define FX_ASM(TAB, BODY)                                                                                           \
+    asm volatile("{\n\t" FX_REGS FX_REGS_S TAB "mov.b32 a0, %0;\n\tmov.b32 a1, %1;\n\tmov.b32 sa, %2;\n\t"           \
+                 "mov.b32 ip, %3;\n\tmov.b32 x0, %4;\n\tmov.b32 x1, %5;\n\tmov.b32 lo, %6;\n\t" FX_START BODY         \
                  "mov.b32 %0, a0;\n\tmov.b32 %1, a1;\n\tmov.b32 %2, sa;\n\tmov.b32 %3, ip;\n\t}"                     \
                  : "+f"(a[0]), "+f"(a[1]), "+r"(sa), "+r"(ip) : "f"(x[0]), "f"(x[1]), "r"(lo) : "memory")
-        if constexpr (V == VF) FX_ASM2(FX_TABLE, FX_BODY_F(2));
-        else if constexpr (V == VI) FX_ASM2(FX_TABLE, FX_BODY_I(2));
-        else FX_ASM2(FX_BTABLE, FX_BODY_B(2));
+        if constexpr (V == VI) FX_ASM(FX_TABLE, FX_BODY_I(S2));
+        else FX_ASM(FX_BTABLE, FX_BODY_B(S2));
+#undef FX_ASM
+    } else if constexpr (K == 2) {
+        asm volatile("{\n\t" FX_REGS FX_REGS_P FX_TABLE "mov.b64 a0, {%0, %1};\n\tmov.b32 sa, %2;\n\tmov.b32 ip, %3;\n\t"
+                     "mov.b64 x0, {%4, %5};\n\t" FX_START FX_BODY_F(P2, "x2")
+                     "mov.b64 {%0, %1}, a0;\n\tmov.b32 %2, sa;\n\tmov.b32 %3, ip;\n\t}"
+                     : "+f"(a[0]), "+f"(a[1]), "+r"(sa), "+r"(ip) : "f"(x[0]), "f"(x[1]) : "memory");
     } else {
         static_assert(K == 4 && V == VF, "four cases per lane: binary32 only");
-        asm volatile("{\n\t" FX_REGS FX_TABLE
-                     "mov.b32 a0, %0;\n\tmov.b32 a1, %1;\n\tmov.b32 a2, %2;\n\tmov.b32 a3, %3;\n\tmov.b32 sa, %4;\n\t"
-                     "mov.b32 ip, %5;\n\tmov.b32 x0, %6;\n\tmov.b32 x1, %7;\n\tmov.b32 x2, %8;\n\tmov.b32 x3, %9;\n\t"
-                     "mov.b32 lo, %10;\n\t" FX_START FX_BODY_F(4)
-                     "mov.b32 %0, a0;\n\tmov.b32 %1, a1;\n\tmov.b32 %2, a2;\n\tmov.b32 %3, a3;\n\tmov.b32 %4, sa;\n\t"
-                     "mov.b32 %5, ip;\n\t}"
+        asm volatile("{\n\t" FX_REGS FX_REGS_P FX_TABLE "mov.b64 a0, {%0, %1};\n\tmov.b64 a1, {%2, %3};\n\t"
+                     "mov.b32 sa, %4;\n\tmov.b32 ip, %5;\n\tmov.b64 x0, {%6, %7};\n\tmov.b64 x1, {%8, %9};\n\t"
+                     FX_START FX_BODY_F(P4, "x2")
+                     "mov.b64 {%0, %1}, a0;\n\tmov.b64 {%2, %3}, a1;\n\tmov.b32 %4, sa;\n\tmov.b32 %5, ip;\n\t}"
                      : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+r"(sa), "+r"(ip)
-                     : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "r"(lo) : "memory");
+                     : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]) : "memory");
     }
 }
 
@@ -339,7 +396,7 @@ struct FxCtx {
     uint32_t lt;         // leaf table (shared address below 64 KB: operands hold two 16-bit addresses)
     uint32_t lo;         // this lane's offset in a row of the Boolean leaf table
     uint32_t W, maxd;    // entries in shared memory, entries in all
-    float* g;            // global overflow: (maxd - W) entries x 32 lanes x K
+    float* g;            // global overflow: maxd entries x 32 lanes x K
     float x[K];          // the lane's inputs (binary32, integer)
 };
 
@@ -348,8 +405,9 @@ struct FxCtx {
 // block, lane by lane, K words per lane; a row is 128 K bytes.
 template <int K, int V>
 struct FxTable {
-    static constexpr int row = 32 * K * 4;                     // bytes of a Boolean row
-    __host__ __device__ static uint32_t bytes(uint32_t ncb) { return V == VB ? FX_BROWS * row * ncb : 1024u; }
+    // bytes of an entry: a Boolean row, a constant (twice at K = 2 and 4: operands of paired instructions)
+    static constexpr int row = V == VB ? 32 * K * 4 : (V == VF && K > 1) ? 8 : 4;
+    __host__ __device__ static uint32_t bytes(uint32_t ncb) { return V == VB ? FX_BROWS * row * ncb : 256u * row; }
     // address of case block cb's table
     __device__ static uint32_t at(uint32_t base, uint32_t cb) { return V == VB ? base + cb * FX_BROWS * row : base; }
     __device__ static void fill(float* tab, const float* consts, uint32_t ncb) {
@@ -360,26 +418,39 @@ struct FxTable {
                 tab[i] = op < 4u ? 0.0f : __uint_as_float(mux_word(b, mux_pattern(b < 5u ? b : 0u), w));
             }
         } else {
-            for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) tab[i] = (i >= 5) ? consts[i - 5] : 0.0f;
+            constexpr uint32_t n = row / 4;
+            for (uint32_t i = threadIdx.x; i < 256 * n; i += blockDim.x) tab[i] = (i / n >= 5) ? consts[i / n - 5] : 0.0f;
         }
     }
 };
 
-// The list at ip on the checked path: entries from W on live in the global
-// overflow area.  sa counts as on the fast path (it is only read through the
-// window).  False when the stack is deeper than maxd.
-template <int K, int V>
-__device__ __forceinline__ bool fx_exec_checked(uint32_t& ip, float (&a)[K], uint32_t& sa, const FxCtx<K>& c) {
+// Slide the window: entries [0, lo) of the stack are in global memory, the
+// others at stack + (i - lo) entries.  Every lane moves its own column.
+template <int K>
+__device__ __forceinline__ void fx_slide(const FxCtx<K>& c, uint32_t& lo, uint32_t& sa, uint32_t to) {
     constexpr uint32_t stride = 32 * K * 4;
-    const int lane = lane_id();
-    uint32_t dep = (sa - c.stack) / stride;
-    bool ok = true;
-    auto push = [&]() {
-        if (dep < c.W) sts_vec<K>(c.stack + dep * stride, a);
-        else if (dep < c.maxd) vstore<K>(c.g + ((size_t)(dep - c.W) * 32 + lane) * K, a);
-        else ok = false;
-        if (dep < c.maxd) ++dep;
-    };
+    float* g = c.g + lane_id() * K;
+    const uint32_t have = (sa - c.stack) / stride;          // entries in the window
+    float v[K];
+    if (to > lo) {
+        const uint32_t n = to - lo;
+        for (uint32_t j = 0; j < n; ++j) { lds_vec<K>(c.stack + j * stride, v); vstore<K>(g + (size_t)(lo + j) * 32 * K, v); }
+        for (uint32_t j = n; j < have; ++j) { lds_vec<K>(c.stack + j * stride, v); sts_vec<K>(c.stack + (j - n) * stride, v); }
+        sa -= n * stride;
+    } else {
+        const uint32_t n = lo - to;
+        for (uint32_t j = have; j-- > 0;) { lds_vec<K>(c.stack + j * stride, v); sts_vec<K>(c.stack + (j + n) * stride, v); }
+        for (uint32_t j = 0; j < n; ++j) { vload<K>(g + (size_t)(to + j) * 32 * K, v); sts_vec<K>(c.stack + j * stride, v); }
+        sa += n * stride;
+    }
+    lo = to;
+}
+
+// The list at ip with the whole stack, `dep` entries, in the global area.
+template <int K, int V>
+__device__ __forceinline__ void fx_exec_global(uint32_t& ip, float (&a)[K], uint32_t& dep, const FxCtx<K>& c) {
+    float* g = c.g + lane_id() * K;
+    auto push = [&]() { vstore<K>(g + (size_t)dep * 32 * K, a); ++dep; };
     auto leaf = [&](uint32_t y, bool cst, float (&v)[K]) {
         if constexpr (V == VB) { lds_vec<K>(y + c.lo, v); (void)cst; }
         else {
@@ -406,20 +477,38 @@ __device__ __forceinline__ bool fx_exec_checked(uint32_t& ip, float (&a)[K], uin
 #pragma unroll
             for (int k = 0; k < K; ++k) a[k] = l[k];
         } else if (idx < 28u) {
-            if (dep) --dep;
-            if (dep < c.W) lds_vec<K>(c.stack + dep * stride, r);
-            else vload<K>(c.g + ((size_t)(dep - c.W) * 32 + lane) * K, r);
+            --dep;
+            vload<K>(g + (size_t)dep * 32 * K, r);
             apply_vec<K, V>(idx - 24u, a, r);
         } else {
-            leaf(y, idx & 1u, l);
             push();
+            leaf(y, idx & 1u, l);
 #pragma unroll
             for (int k = 0; k < K; ++k) a[k] = l[k];
         }
     }
     ip += 8;                       // past the end mark
-    sa = c.stack + dep * stride;
-    return ok;
+}
+
+// Make the window fit the chunk about to run; false when its depths span
+// more than the window (the stack is then all in the global area).  `lo`
+// entries are below the window; an instruction whose leaves lie in the chunk
+// to the right leaves the stack up to two entries short of B.
+template <int K>
+__device__ __forceinline__ bool fx_fit(const FxChunk& ch, const FxCtx<K>& c, uint32_t& lo, uint32_t& sa, bool& ok) {
+    const int32_t top = (int32_t)(lo + c.W);
+    const bool low = lo > 0 && (ch.in < (int32_t)lo + 2 || ch.mn < (int32_t)lo);
+    if (!__any_sync(FULL, ch.in > top || ch.mx > top || low)) return true;
+    const int32_t mx = max(ch.in, __reduce_max_sync(FULL, ch.mx));
+    const int32_t mn = max(0, min(ch.in - 2, __reduce_min_sync(FULL, ch.mn)));
+    if (mx > (int32_t)c.maxd) { ok = false; return true; }
+    const int32_t span = mx - mn;
+    if (span <= (int32_t)c.W) {
+        fx_slide<K>(c, lo, sa, (uint32_t)max(0, mn - ((int32_t)c.W - span) / 2));
+        return true;
+    }
+    fx_slide<K>(c, lo, sa, lo + (sa - c.stack) / (32 * K * 4));
+    return false;
 }
 
 // Evaluate the nodes [s, e): afterwards a holds the value of the subtree at
@@ -438,7 +527,7 @@ __device__ __forceinline__ bool fx_run(LD ld, uint32_t s, uint32_t e, uint32_t w
     cy.rw = 0xFFFFFFFFu;
     cy.rf = 0u;
     cy.B = 0;
-    uint32_t sa = c.stack, wl = w1;
+    uint32_t sa = c.stack, lo = 0, wl = w1;
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = 0.f;
@@ -446,11 +535,13 @@ __device__ __forceinline__ bool fx_run(LD ld, uint32_t s, uint32_t e, uint32_t w
         if (stop && *stop) { *aborted = true; return true; }
         const uint32_t fl = fx_funcs(wl);
         const uint32_t wn = fx_word(ld, base - 2 * FX_CHUNK + 4 * lane, s, e);     // in flight during this chunk
-        const FxChunk ch = fx_decode<V, false, FxTable<K, V>::row>(cy, fl, base, s, e, c.W, c.code, c.lt, 0u);
+        const FxChunk ch = fx_decode<V, false, FxTable<K, V>::row>(cy, fl, base, s, e, c.code, c.lt, 0u);
         if (ch.bad) { ok = false; break; }
         uint32_t ip = c.code;
-        if (!ch.over) fx_exec<K, V>(ip, a, sa, c.x, c.lo);
-        else ok &= fx_exec_checked<K, V>(ip, a, sa, c);
+        const bool fits = fx_fit<K>(ch, c, lo, sa, ok);
+        if (!ok) break;
+        if (fits) fx_exec<K, V>(ip, a, sa, c.x, c.lo);
+        else fx_exec_global<K, V>(ip, a, lo, c);
         __syncwarp();
         if (base <= (int32_t)s) break;
         base -= FX_CHUNK;

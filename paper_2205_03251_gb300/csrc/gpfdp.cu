@@ -750,7 +750,7 @@ int gp_pop_create(const gp_config* cfg_in, const float* x, const float* targets,
         int r = with_kind(d, [&](auto k, auto v) { return setup_items_kernel<decltype(k)::value, decltype(v)::value>(pop); });
         if (r) { g_create_error = pop->err; return bail(r); }
         d.ovf_warps = (uint32_t)pop->grid_items * GP_WARPS;
-        DA2(d.ovf, (size_t)d.ovf_warps * (d.maxdepth - d.W) * 32 * K);
+        DA2(d.ovf, (size_t)d.ovf_warps * d.maxdepth * 32 * K);
     }
     // generation buffers
     {
