@@ -22,7 +22,7 @@ enum : uint32_t {
 };
 
 // queue counters
-enum { Q_ITEMS = 0, Q_SKEL = 1, Q_WALK = 2, Q_MISC = 3, Q_ALLOC = 4, Q_PATHV = 5, Q_WALK_LONG = 6, NQ = 16 };
+enum { Q_ITEMS = 0, Q_SKEL = 1, Q_WALK = 2, Q_WALK_LONG = 6, Q_CLIMB = 7, NQ = 16 };
 
 // Value kinds of the function sets.  Every value travels as 32 bits in a
 // float register or slot: a binary32 number (VF), a word of 32 Boolean
@@ -60,7 +60,8 @@ struct DevPop {
     // items (small subtrees hanging off the cached skeleton)
     uint4* it_desc;      // [Ecap] (start, length, slot, buffer) of the entry's small-subtree item
     uint4* sk_desc;      // [Ecap] (slot, operand slot, op | child flags, right child entry) for the skeleton pass
-    uint32_t* order;     // [Ecap] work order
+    uint32_t* order;     // [Ecap] where the skeleton pass starts: the largest small cached subtrees
+    uint32_t* e_flag;    // [Ecap] skeleton pass: case blocks of which one child's value has arrived
     // values: one pool of slots shared by the parents' and the children's caches
     float* slots;        // [Scap][Cpad]
     uint32_t* live;      // [Scap] generation stamp of the last cache that referenced the slot

@@ -5,9 +5,20 @@
 #pragma once
 #include "fused.cuh"
 
+// Entries a warp of the skeleton pass evaluates by itself before it climbs.
+// (32: bushy trees climb a twentieth of their entries; with four cases per lane shared memory
+// for the values of 8.)
+__host__ __device__ constexpr uint32_t sk_group(uint32_t K) { return K == 4 ? 8u : 32u; }
+// Does entry e's cached subtree (its entries are contiguous) fit a group?
+__device__ __forceinline__ bool sk_small(const DevPop& d, const uint32_t* __restrict__ e_tree, uint32_t e) {
+    const uint32_t x = e + sk_group(d.K);
+    return x >= d.e_off[e_tree[e] + 1] || d.e_pos[x] >= d.e_end[e];
+}
+
 // Work item of entry e: the part of its subtree not covered by large
 // children -- the whole subtree when both children are small, else the
 // small child (its value is parked in e's slot until the skeleton pass).
+// Also the list of entries the skeleton pass starts from (d.order).
 __global__ void k_build_items(DevPop d, const uint32_t* __restrict__ e_tree) {
     if (halted(d)) return;
     const uint32_t ne = d.e_off[d.P];
@@ -24,7 +35,19 @@ __global__ void k_build_items(DevPop d, const uint32_t* __restrict__ e_tree) {
         const uint32_t oslot = (c0 >= 0 && c1 >= 0) ? d.e_slot[c1] : d.e_slot[e];
         d.sk_desc[e] = make_uint4(d.e_slot[e], oslot, op | ((c0 >= 0) ? 0x100u : 0u) | ((c1 >= 0) ? 0x200u : 0u),
                                   (uint32_t)c1);
-        d.order[e] = e;
+        // the climbs of the skeleton pass start at the largest entries whose cached subtree is small
+        d.e_flag[e] = 0u;
+        const int32_t p = d.e_par[e];
+        const uint32_t here = __activemask();
+        const bool start = sk_small(d, e_tree, e) && (p < 0 || !sk_small(d, e_tree, (uint32_t)p));
+        const uint32_t mk = __ballot_sync(here, start);
+        if (start) {
+            const int lead = __ffs(mk) - 1;
+            uint32_t at = 0;
+            if (lane_id() == lead) at = atomicAdd(&d.q[Q_SKEL], (uint32_t)__popc(mk));
+            at = __shfl_sync(mk, at, lead);
+            d.order[at + __popc(mk & ((1u << lane_id()) - 1u))] = e;
+        }
     }
 }
 
@@ -120,90 +143,148 @@ __global__ void __launch_bounds__(GP_WARPS * 32, K == 4 ? 3 : V == VF ? 4 : 5) k
     if (lane == 0 && ops_done) { atomicAdd(&d.acc_ops[0], ops_done); atomicAdd(&d.acc_ops[2], ops_done); }
 }
 
-// Cached nodes bottom up: entries of a tree in decreasing position order,
-// so both children of a node are done before it.  A node with one large
-// child has that child at the next entry index (no other cached node lies
-// between them), a node with two has its left child there.  Entries are
-// taken in groups of SKB: descriptors (prefetched one group ahead) and
-// operand vectors are loaded first -- they do not depend on the running
-// value -- then combined in order; a right child inside the same group is
-// taken from the group's own results.
-#define SKB 16
+// Cached nodes bottom up.  A warp (per case block) first evaluates a whole
+// small cached subtree, up to sk_group entries, from its last entry to its
+// first: a node's left or only cached child is the next entry, whose value is
+// the running one, its right one was computed earlier and waits in shared
+// memory, and the items' values it combines with depend on nothing, so they
+// are loaded SKB at a time.  Then it climbs.  The run of nodes with one cached
+// child above an entry is a run of descending indexes: their descriptors come
+// in one load of 32.  At a node with two cached children the warp that
+// arrives first leaves its value in the slot and ends; the second one
+// combines both and goes on (a bit per node and case block, set by atomicOr).
+// No warp waits.  Bound by latency along a tree's longest chain; every chain
+// and case block runs at once, where a warp per tree took the chains and the
+// case blocks one after another: 500 grafted trees of ~1e6 nodes x 48 cases
+// 1.10 -> 0.43 ms, 1,500 uneven trees over the 11-multiplexer 1.06 -> 0.38 ms,
+// 600 uneven trees x 1,000 cases 14.2 -> 0.67 ms.  cb0, ncbp: the case blocks
+// of this launch (at most 32, the bits of a flag word).
+#define SKB 8
+#define SK_WARPS 4
 template <int K, int V>
-__global__ void __launch_bounds__(GP_WARPS * 32) k_eval_skeleton(DevPop d) {
+__global__ void __launch_bounds__(SK_WARPS * 32) k_eval_skeleton(DevPop d, uint32_t cb0, uint32_t ncbp) {
     if (halted(d)) return;
-    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
+    __shared__ __align__(16) float done[SK_WARPS][sk_group(K)][32 * K];           // values of the group's entries
     const int lane = lane_id();
-    if (d.e_off[d.P] > d.Ecap) return;
-    for (uint32_t tree = gw; tree < d.P; tree += nw) {
-        const uint32_t e0 = d.e_off[tree], e1 = d.e_off[tree + 1];
-        unsigned long long cnt = 0;
-        for (uint32_t cbk = 0; cbk < d.ncb; ++cbk) {
-            float prev[K];
+    const uint32_t ne = d.e_off[d.P];
+    if (ne > d.Ecap) return;
+    const uint32_t nunits = d.q[Q_SKEL] * ncbp, nwarps = gridDim.x * SK_WARPS;
+    float (*mine)[32 * K] = done[threadIdx.x >> 5];
+    uint32_t cnt = 0;
+    // Units from a queue, each taken when the warp is free: a unit taken ahead
+    // would be held up by the climb before it, and every unit above would wait.
+    uint32_t u = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    while (u < nunits) {
+        const uint32_t cb = u % ncbp, cbk = cb0 + cb;
+        uint32_t e = d.order[u / ncbp];
+        float val[K];
+        uint4 gd = make_uint4(0, 0, 0, 0);
+        uint32_t pos = 0xFFFFFFFFu, tree = 0;
+        const uint32_t x = e + lane, end = d.e_end[e];
+        if (lane < (int)sk_group(K) && x < ne) { gd = d.sk_desc[x]; pos = d.e_pos[x]; tree = d.e_tree[x]; }
+        const uint32_t own = __shfl_sync(FULL, tree, 0);
+        const uint32_t n = __popc(__ballot_sync(FULL, pos < end && tree == own));
+        uint4 md = make_uint4(0, 0, 0, 0);                                   // the entries below e: lane l has e - 1 - l
+        if ((uint32_t)lane < e) md = d.sk_desc[e - 1 - lane];
 #pragma unroll
-            for (int k = 0; k < K; ++k) prev[k] = 0.f;
-            uint4 md = make_uint4(0, 0, 0, 0);
-            if (e1 > e0 && lane < SKB && (uint32_t)lane < e1 - e0) md = d.sk_desc[e1 - 1 - lane];
-            for (uint32_t top = e1; top > e0;) {
-                const uint32_t nb = (top - e0 < SKB) ? top - e0 : SKB;
-                const uint32_t ntop = top - nb;
-                uint4 mdn = make_uint4(0, 0, 0, 0);
-                if (ntop > e0 && lane < SKB && (uint32_t)lane < ntop - e0) mdn = d.sk_desc[ntop - 1 - lane];
-                float opnd[SKB][K];
-                uint32_t slots[SKB], info[SKB], c1s[SKB];
+        for (int k = 0; k < K; ++k) val[k] = 0.f;
+        for (int top = (int)n; top > 0; top -= SKB) {
+            float opnd[SKB][K];
 #pragma unroll
-                for (int j = 0; j < SKB; ++j) {
-                    slots[j] = __shfl_sync(FULL, md.x, j);
-                    const uint32_t os = __shfl_sync(FULL, md.y, j);
-                    info[j] = __shfl_sync(FULL, md.z, j);
-                    c1s[j] = __shfl_sync(FULL, md.w, j);
-                    if (j < (int)nb) load_slot<K>(d, os, cbk, opnd[j]);
-                }
-                float done[SKB][K];
+            for (int j = 0; j < SKB; ++j) {
+                const uint32_t os = __shfl_sync(FULL, gd.y, top - 1 - j);
+                const uint32_t info = __shfl_sync(FULL, gd.z, top - 1 - j);
+                if (top - 1 - j >= 0 && (info & 0x300u) != 0x300u) load_slot<K>(d, os, cbk, opnd[j]);
+            }
 #pragma unroll
-                for (int j = 0; j < SKB; ++j) {
-                    if (j < (int)nb) {
-                        const bool has0 = info[j] & 0x100u, has1 = info[j] & 0x200u;
-                        const uint32_t op = info[j] & 0xFFu;
-                        float val[K];
-                        if (!has0 && !has1) {
+            for (int j = 0; j < SKB; ++j) {
+                const int l = top - 1 - j;
+                const uint32_t info = __shfl_sync(FULL, gd.z, l), slot = __shfl_sync(FULL, gd.x, l);
+                const uint32_t right = __shfl_sync(FULL, gd.w, l) - e;
+                if (l >= 0) {
+                    if ((info & 0x300u) == 0u) {                             // an item's value
 #pragma unroll
-                            for (int k = 0; k < K; ++k) val[k] = opnd[j][k];
-                        } else {
-                            float o[K];
+                        for (int k = 0; k < K; ++k) val[k] = opnd[j][k];
+                    } else {
+                        if ((info & 0x300u) == 0x300u) vload<K>(&mine[right][lane * K], opnd[j]);
+                        else if (!(info & 0x100u)) {                         // the running value is the right operand
 #pragma unroll
-                            for (int k = 0; k < K; ++k) o[k] = opnd[j][k];
-                            if (has0 && has1) {
-#pragma unroll
-                                for (int jj = 0; jj < j; ++jj)
-                                    if (c1s[j] == top - 1 - jj) {
-#pragma unroll
-                                        for (int k = 0; k < K; ++k) o[k] = done[jj][k];
-                                    }
-                            }
-                            if (has0) {                       // left = entry e+1 = prev
-#pragma unroll
-                                for (int k = 0; k < K; ++k) val[k] = prev[k];
-                                apply_vec<K, V>(op, val, o);
-                            } else {                          // right = entry e+1 = prev
-#pragma unroll
-                                for (int k = 0; k < K; ++k) val[k] = o[k];
-                                apply_vec<K, V>(op, val, prev);
-                            }
-                            store_slot<K>(d, slots[j], cbk, val);
-                            if (cbk == 0) ++cnt;
+                            for (int k = 0; k < K; ++k) { const float t = val[k]; val[k] = opnd[j][k]; opnd[j][k] = t; }
                         }
-#pragma unroll
-                        for (int k = 0; k < K; ++k) { done[j][k] = val[k]; prev[k] = val[k]; }
+                        apply_vec<K, V>(info & 0xFFu, val, opnd[j]);
+                        store_slot<K>(d, slot, cbk, val);
+                        if (cbk == 0) ++cnt;
                     }
+                    vstore<K>(&mine[l][lane * K], val);
                 }
-                top = ntop;
-                md = mdn;
             }
         }
-        if (lane == 0 && cnt) atomicAdd(&d.acc_ops[0], cnt);
+        for (;;) {
+            // the run of nodes with one cached child above e
+            const bool h0 = md.z & 0x100u, h1 = md.z & 0x200u;
+            const uint32_t other = __ballot_sync(FULL, h0 == h1);            // none or two: the run ends
+            const uint32_t run = other ? (uint32_t)__ffs(other) - 1u : 32u;
+            const int32_t up = run < 32u ? d.e_par[e - run] : 0;             // (needed after the run)
+            for (uint32_t j0 = 0; j0 < run; j0 += SKB) {
+                float opnd[SKB][K];
+#pragma unroll
+                for (int j = 0; j < SKB; ++j) {
+                    const uint32_t os = __shfl_sync(FULL, md.y, (int)j0 + j);
+                    if (j0 + j < run) load_slot<K>(d, os, cbk, opnd[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < SKB; ++j) {
+                    const uint32_t info = __shfl_sync(FULL, md.z, (int)j0 + j), slot = __shfl_sync(FULL, md.x, (int)j0 + j);
+                    if (j0 + j < run) {
+                        if (!(info & 0x100u)) {                              // the running value is the right operand
+#pragma unroll
+                            for (int k = 0; k < K; ++k) { const float t = val[k]; val[k] = opnd[j][k]; opnd[j][k] = t; }
+                        }
+                        apply_vec<K, V>(info & 0xFFu, val, opnd[j]);
+                        store_slot<K>(d, slot, cbk, val);
+                    }
+                }
+            }
+            e -= run;
+            if (cbk == 0) cnt += run;                       // nodes combined, once
+            if (run == 32) {
+                md = make_uint4(0, 0, 0, 0);
+                if ((uint32_t)lane < e) md = d.sk_desc[e - 1 - lane];
+                continue;
+            }
+            // e's parent has two cached children (e the left one when it is the entry before e), or e is a root
+            const uint32_t below = __shfl_sync(FULL, md.z, (int)run);
+            const bool left = (below & 0x300u) == 0x300u;
+            const int32_t p = left ? (int32_t)e - 1 : up;
+            if (p < 0) break;
+            // all that the second to arrive needs but the value, loaded before it is known who that is
+            const uint32_t info = left ? below : d.sk_desc[p].z;
+            const uint32_t slot = left ? __shfl_sync(FULL, md.x, (int)run) : d.sk_desc[p].x;
+            const uint32_t sib = left ? __shfl_sync(FULL, md.y, (int)run) : d.sk_desc[p + 1].x;
+            md = make_uint4(0, 0, 0, 0);
+            if (lane < p) md = d.sk_desc[p - 1 - lane];
+            uint32_t first = 0;
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) first = !(atomicOr(&d.e_flag[p], 1u << cb) & (1u << cb));
+            if (__shfl_sync(FULL, first, 0)) break;
+            __threadfence();
+            float o[K];
+            load_slot<K>(d, sib, cbk, o);
+            if (!left) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) { const float t = val[k]; val[k] = o[k]; o[k] = t; }
+            }
+            apply_vec<K, V>(info & 0xFFu, val, o);
+            store_slot<K>(d, slot, cbk, val);
+            e = (uint32_t)p;
+            if (cbk == 0) ++cnt;
+        }
+        __syncwarp();
+        if (lane == 0) u = nwarps + atomicAdd(&d.q[Q_CLIMB], 1u);
+        u = __shfl_sync(FULL, u, 0);
     }
+    if (lane == 0 && cnt) atomicAdd(&d.acc_ops[0], (unsigned long long)cnt);
 }
 
 // Fitness of every tree from its root's cached vector (a warp per tree).

@@ -66,7 +66,6 @@ struct GenBufs {
     uint32_t* nins;                  // [P] child-cached nodes the mother does not cache (inserted entries)
     uint4* mb;                       // [P] merge bounds: first mother entry >= c, >= c+r, father >= d, >= d+s
     uint32_t* mcnt;                  // [P+1] children's entry counts, then offsets
-    uint32_t* src;                   // [Ecap] value source of each child entry (bit 31: walk record)
     uint32_t* pv_cnt;                // [P]
     uint32_t* pv_off;                // [P+1]
     uint4* pv_sorted;                // [pvcap] (pos, slot | insert<<31, child end, 0), per child in walk order
@@ -2275,7 +2274,6 @@ __device__ __forceinline__ void put_entry(const DevPop& d, GenBufs& g, uint32_t 
     d.e_c1[x] = -1;
     d.e_par[x] = -1;
     d.e_slot[x] = (src & 0x80000000u) ? SLOT_NEW : src;
-    g.src[x] = src;
     if (src & 0x80000000u) g.rec_entry[src & 0x7FFFFFFFu] = x;
 }
 

@@ -35,7 +35,7 @@ constexpr int NREC = 128;   // event pairs kept per phase: stats average the las
 // set is built.
 struct CacheSet {
     uint32_t *e_cnt = nullptr, *e_off = nullptr, *e_pos = nullptr, *e_end = nullptr, *e_slot = nullptr;
-    uint32_t *order = nullptr, *e_tree = nullptr, *e_cmax = nullptr, *msrc = nullptr;
+    uint32_t *order = nullptr, *e_tree = nullptr, *e_cmax = nullptr, *e_flag = nullptr;
     int32_t *e_par = nullptr, *e_c0 = nullptr, *e_c1 = nullptr, *e_bal = nullptr;
     uint4 *it_desc = nullptr, *sk_desc = nullptr;
     uint32_t Ecap = 0;
@@ -52,7 +52,7 @@ struct gp_pop {
     StructBufs sb;
     GenBufs gb;
     int dev, nsm;
-    int grid_items, grid_warps, grid_threads;
+    int grid_items, grid_skel, grid_warps, grid_threads;
     size_t smem_items;
     std::string err;
     gp_stats stats;
@@ -286,6 +286,8 @@ int setup_items_kernel(gp_pop* pop) {
     if (nb < 1) nb = 1;
     pop->grid_items = nb * pop->nsm;
     pop->smem_items = smem;
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_eval_skeleton<K, V>, SK_WARPS * 32, 0));
+    pop->grid_skel = (nb < 1 ? 1 : nb) * pop->nsm;
     // the one-pass interpreter: CTAs of OP_EVAL_WARPS warps, as many as fit
     // (at most OP_CTAS_PER_SM per SM), each warp with its own overflow stack
     const size_t smem_op = OnePassEvalLayout<K>::total((int)pop->d.W);
@@ -373,13 +375,36 @@ int setup_walk_kernel(gp_pop* pop, uint32_t team) {
     return GP_OK;
 }
 
+// Do the kernels with four cases per lane fit a CTA's shared memory, with
+// this stack window and walk team?
+bool wide_fits(const gp_config& cfg) {
+    int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    const int W = cfg.stack_window ? (int)cfg.stack_window : 16;
+    const uint32_t ncb = (cfg.n_cases + 127) / 128, team = cfg.walk_team ? cfg.walk_team : 4u;
+    return ItemsLayout<4, VF>::total(W, ncb) <= (size_t)optin && OnePassEvalLayout<4>::total(W) <= (size_t)optin &&
+           TeamLayout<4>(W, ncb * 128, team).total <= (size_t)optin;
+}
+
 template <int K, int V>
 void launch_items(gp_pop* pop) {
     k_eval_items<K, V><<<pop->grid_items, GP_WARPS * 32, pop->smem_items, pop->stream>>>(pop->d);
 }
 template <int K, int V>
 void launch_skeleton(gp_pop* pop) {
-    k_eval_skeleton<K, V><<<pop->grid_warps, GP_WARPS * 32, 0, pop->stream>>>(pop->d);
+    // the flag words have room for 32 case blocks: more go in further launches
+    for (uint32_t cb0 = 0; cb0 < pop->d.ncb; cb0 += 32) {
+        const uint32_t n = pop->d.ncb - cb0 < 32u ? pop->d.ncb - cb0 : 32u;
+        if (cb0) {
+            cudaMemsetAsync(pop->d.e_flag, 0, sizeof(uint32_t) * pop->d.Ecap, pop->stream);
+            cudaMemsetAsync(pop->d.q + Q_CLIMB, 0, sizeof(uint32_t), pop->stream);
+        }
+        k_eval_skeleton<K, V><<<pop->grid_skel, SK_WARPS * 32, 0, pop->stream>>>(pop->d, cb0, n);
+    }
 }
 
 // Advance the generation offset of a captured generation loop (last node of the graph).
@@ -407,11 +432,10 @@ void bind_set(gp_pop* pop) {
     CacheSet& c = pop->sets[pop->cur];
     d.e_cnt = c.e_cnt; d.e_off = c.e_off; d.e_pos = c.e_pos; d.e_end = c.e_end; d.e_par = c.e_par;
     d.e_c0 = c.e_c0; d.e_c1 = c.e_c1; d.e_slot = c.e_slot; d.e_tree = c.e_tree; d.it_desc = c.it_desc;
-    d.sk_desc = c.sk_desc; d.order = c.order; d.Ecap = c.Ecap;
+    d.sk_desc = c.sk_desc; d.order = c.order; d.e_flag = c.e_flag; d.Ecap = c.Ecap;
     d.slots = pop->pool; d.live = pop->live; d.freeslot = pop->freeslot; d.ftile = pop->ftile;
     d.Scap = (uint32_t)pop->pool_cap;
     pop->sb.e_bal = c.e_bal; pop->sb.e_tree = c.e_tree; pop->sb.e_cmax = c.e_cmax;
-    pop->gb.src = c.msrc;
 }
 
 CacheView view_of(const gp_pop* pop, const CacheSet& c) {
@@ -479,7 +503,7 @@ int grow_set(gp_pop* pop, int which, uint32_t ecap) {
     bool ok = al(&c.e_cnt, d.P + 1) && al(&c.e_off, d.P + 1) && al(&c.e_pos, ecap) && al(&c.e_end, ecap) &&
               al(&c.e_par, ecap) && al(&c.e_c0, ecap) && al(&c.e_c1, ecap) && al(&c.e_slot, ecap) &&
               al(&c.it_desc, ecap) && al(&c.sk_desc, ecap) && al(&c.order, ecap) && al(&c.e_bal, ecap) &&
-              al(&c.e_tree, ecap) && al(&c.e_cmax, ecap / 32 + 2) && al(&c.msrc, ecap);
+              al(&c.e_tree, ecap) && al(&c.e_cmax, ecap / 32 + 2) && al(&c.e_flag, ecap);
     if (!ok) return fail(pop, GP_ENOMEM, "allocation of a cache of %u entries failed", ecap);
     cudaMemset(c.e_off, 0, sizeof(uint32_t) * (d.P + 1));
     c.Ecap = ecap;
@@ -586,7 +610,8 @@ int gp_pop_create(const gp_config* cfg_in, const float* x, const float* targets,
     if (cfg.tournament == 0) cfg.tournament = 7;
     if (cfg.cache_budget_bytes == 0) cfg.cache_budget_bytes = 40ull << 30;
     uint32_t K = cfg.cases_per_lane;
-    if (K == 0) K = (cfg.n_cases <= 32) ? 1 : 2;
+    const bool auto_k = K == 0;
+    if (auto_k) K = (cfg.n_cases <= 32) ? 1 : 2;
     if (K != 1 && K != 2 && K != 4) return fail(nullptr, GP_EINVAL, "cases_per_lane must be 0, 1, 2 or 4");
     if (K == 4 && cfg.funcset != GP_FP32_ARITH)
         return fail(nullptr, GP_EINVAL, "cases_per_lane 4 is for the binary32 set only");
@@ -600,6 +625,9 @@ int gp_pop_create(const gp_config* cfg_in, const float* x, const float* targets,
     if (cfg.arena_buffers && (!cfg.lazy_children || cfg.arena_buffers <= cfg.pop_size ||
                               cfg.arena_buffers > 2 * cfg.pop_size))
         return fail(nullptr, GP_EINVAL, "arena_buffers must be 0, or in (pop_size, 2 x pop_size] with lazy_children");
+    // binary32 cases beyond one block of 64: four to a lane when that pads no further (an instruction's branch then
+    // serves 128 cases) and the kernels' shared memory has room
+    if (auto_k && cfg.funcset == GP_FP32_ARITH && cfg.n_cases > 64 && ((cfg.n_cases - 1) / 64) % 2 == 1 && wide_fits(cfg)) K = 4;
     const uint32_t P = cfg.pop_size;
     for (uint32_t i = 0; i < P; ++i) {
         if (offsets[i + 1] < offsets[i]) return fail(nullptr, GP_EINVAL, "offsets not increasing at %u", i);
