@@ -494,14 +494,19 @@ __device__ __forceinline__ void fx_exec_global(uint32_t& ip, float (&a)[K], uint
 // more than the window (the stack is then all in the global area).  `lo`
 // entries are below the window; an instruction whose leaves lie in the chunk
 // to the right leaves the stack up to two entries short of B.
-template <int K>
-__device__ __forceinline__ bool fx_fit(const FxChunk& ch, const FxCtx<K>& c, uint32_t& lo, uint32_t& sa, bool& ok) {
+// need(): called before the global area is first used; false when there is none.
+struct FxHave {
+    __device__ bool operator()() const { return true; }
+};
+template <int K, typename NEED>
+__device__ __forceinline__ bool fx_fit(const FxChunk& ch, const FxCtx<K>& c, uint32_t& lo, uint32_t& sa, bool& ok,
+                                       NEED& need) {
     const int32_t top = (int32_t)(lo + c.W);
     const bool low = lo > 0 && (ch.in < (int32_t)lo + 2 || ch.mn < (int32_t)lo);
     if (!__any_sync(FULL, ch.in > top || ch.mx > top || low)) return true;
     const int32_t mx = max(ch.in, __reduce_max_sync(FULL, ch.mx));
     const int32_t mn = max(0, min(ch.in - 2, __reduce_min_sync(FULL, ch.mn)));
-    if (mx > (int32_t)c.maxd) { ok = false; return true; }
+    if (mx > (int32_t)c.maxd || !need()) { ok = false; return true; }
     const int32_t span = mx - mn;
     if (span <= (int32_t)c.W) {
         fx_slide<K>(c, lo, sa, (uint32_t)max(0, mn - ((int32_t)c.W - span) / 2));
@@ -516,9 +521,10 @@ __device__ __forceinline__ bool fx_fit(const FxChunk& ch, const FxCtx<K>& c, uin
 // are this lane's words of the last chunk and of the one to its left, read
 // by the caller (fx_first), who can have them in flight early.  `stop`: a
 // shared word that, once nonzero, ends the run early with *aborted set.
-template <int K, int V, typename LD>
+template <int K, int V, typename LD, typename NEED = FxHave>
 __device__ __forceinline__ bool fx_run(LD ld, uint32_t s, uint32_t e, uint32_t w0, uint32_t w1, const FxCtx<K>& c,
-                                       float (&a)[K], const volatile uint32_t* stop = nullptr, bool* aborted = nullptr) {
+                                       float (&a)[K], NEED need = NEED(), const volatile uint32_t* stop = nullptr,
+                                       bool* aborted = nullptr) {
     const int lane = lane_id();
     int32_t base = (int32_t)((e - 1) & ~(uint32_t)(FX_CHUNK - 1));
     FxCarry cy;
@@ -538,7 +544,7 @@ __device__ __forceinline__ bool fx_run(LD ld, uint32_t s, uint32_t e, uint32_t w
         const FxChunk ch = fx_decode<V, false, FxTable<K, V>::row>(cy, fl, base, s, e, c.code, c.lt, 0u);
         if (ch.bad) { ok = false; break; }
         uint32_t ip = c.code;
-        const bool fits = fx_fit<K>(ch, c, lo, sa, ok);
+        const bool fits = fx_fit<K>(ch, c, lo, sa, ok, need);
         if (!ok) break;
         if (fits) fx_exec<K, V>(ip, a, sa, c.x, c.lo);
         else fx_exec_global<K, V>(ip, a, lo, c);

@@ -24,23 +24,25 @@
 #include <mutex>
 
 #include "common.cuh"
-#include "interp.cuh"
+#include "fused.cuh"
 
 namespace {
 
-constexpr int NA_K = 2;                       // test cases per lane (64 per case block)
-constexpr int NA_W = 16;                      // stack entries kept in shared memory per warp
 constexpr int NA_MAX_NODES = 1023;            // largest tree: at most 512 leaves, so the stack
-constexpr int NA_MAXD = NA_W + 520;           //   never holds more than 514 entries
-constexpr int NA_WARPS = 4;                   // warps per CTA
-constexpr int NA_CTAS = 16;                   // persistent CTAs
-constexpr size_t NA_OVF_FLOATS = (size_t)NA_CTAS * NA_WARPS * (NA_MAXD - NA_W) * 32 * NA_K;
-constexpr size_t NA_SCRATCH_FLOATS = NA_OVF_FLOATS + 64;   // overflow stacks, then counters
+constexpr int NA_MAXD = 520;                  //   never holds more than 514 entries
+constexpr int NA_WARPS = 16;                  // warps per CTA, a CTA per SM: what the interpreter's branches need
+constexpr int NA_WIN_FLOATS = 96 * 32;        // a warp's stack window: 96 / K entries
+constexpr int NA_SLOTS = 64;                  // overflow stacks
+constexpr size_t NA_OVF_FLOATS = (size_t)NA_SLOTS * NA_MAXD * 32 * 2;
+constexpr size_t NA_SCRATCH_FLOATS = NA_OVF_FLOATS + 64;   // overflow stacks, then control words
+constexpr uint32_t NA_SPIN = 1u << 22;        // bound on the polls for an overflow stack
+// control words: 0 work counter, 1 status, 2 and 3 overflow stacks in use
 }  // namespace
 
-// The scratch: overflow stacks of the 64 resident warps (8.5 MB: 520 entries
-// x 32 lanes x 2 cases x 4 bytes each), followed by the work counter and the
-// status word.
+// The scratch: 64 overflow stacks (8.5 MB: 520 entries x 32 lanes x 2 cases x
+// 4 bytes each) and the control words.  Any warp may run; one whose tree is
+// deeper than its window in shared memory takes an overflow stack until that
+// tree is done.
 static __device__ __align__(256) float g_noalloc_scratch[NA_SCRATCH_FLOATS];
 
 namespace {
@@ -59,82 +61,125 @@ struct NaArgs {
     float* scratch;       // device address of g_noalloc_scratch
 };
 
-__global__ void __launch_bounds__(NA_WARPS * 32) k_eval_small_noalloc(NaArgs a) {
-    // one block of shared memory: four stack entries of room below the first
-    // stack (the interpreter's fast path may touch them on a malformed tree)
-    struct NaSmem {
-        float pad[4 * 32 * NA_K];
-        float kc[256];
-        float sstack[NA_WARPS][NA_W * 32 * NA_K];
-        uint8_t stage[NA_WARPS][STAGE_BYTES];
-    };
-    __shared__ __align__(16) NaSmem sm;
-    float* const kc = sm.kc;
-    float (*const sstack)[NA_W * 32 * NA_K] = sm.sstack;
-    uint8_t (*const stage)[STAGE_BYTES] = sm.stage;
+template <int K>
+struct NaLayout {
+    static constexpr uint32_t table = FxTable<K, VF>::row * 256;
+    static constexpr uint32_t warp_bytes = NA_WIN_FLOATS * 4 + FX_CODE_BYTES;
+    static constexpr uint32_t total = table + NA_WARPS * warp_bytes;
+};
+
+// A warp per tree (all of its case blocks in turn: the fitness sums them in
+// case order), or, when there are fewer trees than CTAs, a CTA per tree with
+// its warps on the case blocks.  The first trees go round the CTAs, so that a
+// few trees run on as many SMs; the others come from the counter.  3,000
+// uneven trees of up to 1,023 nodes x 100 cases: 2,591 us with 64 warps on
+// the whole chip, 133 us with 16 on each SM.
+template <int K>
+__global__ void __launch_bounds__(NA_WARPS * 32) k_eval_small_noalloc(NaArgs a, uint32_t by_cta) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
-    fill_kc(kc, a.consts);
+    FxTable<K, VF>::fill(reinterpret_cast<float*>(smem_raw), a.consts, 1);
     __syncthreads();
-    uint32_t* counter = reinterpret_cast<uint32_t*>(a.scratch + NA_OVF_FLOATS);
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    const uint32_t wb = sm + NaLayout<K>::table + warp * NaLayout<K>::warp_bytes;
+    volatile uint32_t* ctl = reinterpret_cast<volatile uint32_t*>(a.scratch + NA_OVF_FLOATS);
+    uint32_t* counter = const_cast<uint32_t*>(ctl);
     uint32_t* status = counter + 1;
-    Ictx<NA_K> c;
-    c.s = sstack[warp];
-    c.g = a.scratch + (size_t)(blockIdx.x * NA_WARPS + warp) * (NA_MAXD - NA_W) * 32 * NA_K;
-    c.kc = kc;
-    c.W = NA_W;
+    FxCtx<K> c;
+    c.stack = wb + lane * K * 4;
+    c.code = wb + NA_WIN_FLOATS * 4;
+    c.lt = sm;
+    c.lo = 0;
+    c.W = 96 / K;
     c.maxd = NA_MAXD;
-    const uint32_t ncb = (a.n_cases + 32 * NA_K - 1) / (32 * NA_K);
-    for (;;) {
-        uint32_t i = 0;
-        if (lane == 0) i = atomicAdd(counter, 1u);
-        i = __shfl_sync(FULL, i, 0);
-        if (i >= a.n_trees) break;
+    c.g = nullptr;
+    int held = -1;
+    // An overflow stack.  Its holder never waits for anything, so one comes
+    // free; the wait is bounded all the same.
+    auto need = [&]() -> bool {
+        if (held >= 0) return true;
+        int got = -1;
+        if (lane == 0) {
+            for (uint32_t spin = 0; spin < NA_SPIN && got < 0; ++spin) {
+                for (int w = 0; w < NA_SLOTS / 32 && got < 0; ++w) {
+                    const uint32_t freeb = ~ctl[2 + w];
+                    if (!freeb) continue;
+                    const int bit = __ffs(freeb) - 1;
+                    if (!(atomicOr(counter + 2 + w, 1u << bit) & (1u << bit))) got = 32 * w + bit;
+                }
+                if (got < 0) __nanosleep(64);
+            }
+            if (got < 0) atomicOr(status, 4u);
+            __threadfence();
+        }
+        held = __shfl_sync(FULL, got, 0);
+        if (held >= 0) c.g = a.scratch + (size_t)held * NA_MAXD * 32 * 2;
+        return held >= 0;
+    };
+    auto release = [&]() {
+        if (held < 0) return;
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicAnd(counter + 2 + held / 32, ~(1u << (held & 31)));
+        held = -1;
+    };
+    const uint32_t ncb = (a.n_cases + 32 * K - 1) / (32 * K);
+    const uint32_t first = by_cta ? 1u : (uint32_t)NA_WARPS;        // trees a CTA starts with
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(a.ops);
+    uint32_t i = by_cta ? blockIdx.x : warp * gridDim.x + blockIdx.x;
+    while (i < a.n_trees) {
         const uint64_t s64 = a.off[i], e64 = a.off[i + 1];
         const uint64_t n = e64 - s64;
         // ops_bytes is a multiple of 16, so e64 <= ops_bytes also keeps the
-        // staged 16-byte chunks inside the buffer (no rounding that could wrap)
-        if (e64 < s64 || n == 0 || n > NA_MAX_NODES || e64 > a.ops_bytes) {
-            if (lane == 0) atomicOr(status, 1u);
-            continue;
-        }
-        // stage the tree: aligned 16-byte chunks relative to the (16-aligned) ops base
-        const uint32_t s = (uint32_t)(s64 & 15u), e = s + (uint32_t)n;
-        __syncwarp();
-        stage_issue(stage[warp], a.ops + (s64 & ~15ull), s, e);
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncwarp();
+        // words read inside the buffer (no rounding that could wrap)
+        const bool fits = e64 >= s64 && n != 0 && n <= NA_MAX_NODES && e64 <= a.ops_bytes;
+        if (!fits && lane == 0) atomicOr(status, 1u);
         float fit = 0.0f;
-        for (uint32_t cb = 0; cb < ncb; ++cb) {
+        if (fits) {
+            const uint32_t s = (uint32_t)(s64 & 3u), e = s + (uint32_t)n;
+            const uint32_t* tree = words + (s64 >> 2);
+            auto ld = [&](uint32_t q) { return __ldg(tree + (q >> 2)); };
+            for (uint32_t cb = by_cta ? warp : 0; cb < ncb; cb += by_cta ? NA_WARPS : 1) {
+                // lanes past the last case repeat it: their values are not written
 #pragma unroll
-            for (int k = 0; k < NA_K; ++k) {
-                const uint32_t cc = cb * 32 * NA_K + k * 32 + lane;
-                c.xv[k] = (cc < a.n_cases) ? a.x[cc] : 0.0f;
-            }
-            Istate<NA_K> st;
+                for (int k = 0; k < K; ++k) c.x[k] = a.x[min(cb * 32 * K + k * 32 + lane, a.n_cases - 1)];
+                uint32_t w0, w1;
+                fx_first(ld, s, e, w0, w1);
+                float v[K];
+                bool ok = fx_run<K, VF>(ld, s, e, w0, w1, c, v, need);
+                if (!ok && lane == 0) atomicOr(status, 2u);
 #pragma unroll
-            for (int k = 0; k < NA_K; ++k) st.acc[k] = 0.f;
-            st.sp = 0;
-            st.ok = true;
-            interp_staged<NA_K>(stage[warp], s, e, st, c);
-            if (!__all_sync(FULL, st.ok)) { if (lane == 0) atomicOr(status, 2u); }
-#pragma unroll
-            for (int k = 0; k < NA_K; ++k) {
-                const uint32_t cc = cb * 32 * NA_K + k * 32 + lane;
-                if (cc < a.n_cases) a.values[(size_t)i * a.n_cases + cc] = st.acc[k];
-            }
-            __syncwarp();
-            // fitness in case order: lane 0 walks this block's cases through the warp
-#pragma unroll
-            for (int k = 0; k < NA_K; ++k) {
-                for (int l = 0; l < 32; ++l) {
-                    const float v = __shfl_sync(FULL, st.acc[k], l);
-                    const uint32_t cc = cb * 32 * NA_K + k * 32 + l;
-                    if (lane == 0 && cc < a.n_cases) fit = __fadd_rn(fit, fabsf(__fsub_rn(v, a.t[cc])));
+                for (int k = 0; k < K; ++k) {
+                    const uint32_t cc = cb * 32 * K + k * 32 + lane;
+                    const bool in = cc < a.n_cases;
+                    if (in) a.values[(size_t)i * a.n_cases + cc] = v[k];
+                    if (!by_cta) {
+                        // fitness in case order: the terms of 32 cases at once, then their sum
+                        const float term = in ? fabsf(__fsub_rn(v[k], a.t[cc])) : 0.0f;
+                        const uint32_t m = min(32u, a.n_cases - min(a.n_cases, cb * 32 * K + k * 32));
+                        for (uint32_t l = 0; l < m; ++l) fit = __fadd_rn(fit, __shfl_sync(FULL, term, l));
+                    }
                 }
             }
+            release();
         }
-        if (lane == 0) a.fitness[i] = fit;
+        if (by_cta) {
+            __syncthreads();                        // the tree's values, all of its case blocks
+            if (warp == 0 && fits)
+                for (uint32_t b = 0; b < a.n_cases; b += 32) {
+                    const uint32_t j = b + lane, m = min(32u, a.n_cases - b);
+                    const float term = j < a.n_cases ? fabsf(__fsub_rn(a.values[(size_t)i * a.n_cases + j], a.t[j])) : 0.0f;
+                    for (uint32_t l = 0; l < m; ++l) fit = __fadd_rn(fit, __shfl_sync(FULL, term, l));
+                }
+        }
+        if (fits && lane == 0 && (!by_cta || warp == 0)) a.fitness[i] = fit;
+        if (by_cta) {
+            i += gridDim.x;                         // (by_cta: at most one tree per CTA)
+        } else {
+            uint32_t v = 0;
+            if (lane == 0) v = atomicAdd(counter, 1u);
+            i = gridDim.x * first + __shfl_sync(FULL, v, 0);
+        }
     }
 }
 
@@ -144,6 +189,7 @@ std::mutex g_na_mu;
 // the module again, so the address is looked up again in the new context
 float* g_na_ptr[64] = {};
 void* g_na_ctx[64] = {};
+int g_na_nsm[64] = {};
 
 // the current context through the driver entry point (no link-time
 // dependency on the driver library)
@@ -178,6 +224,7 @@ extern "C" int gp_eval_small_noalloc(const uint8_t* d_ops, size_t ops_bytes, con
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return GP_ECUDA;
     float* scratch = nullptr;
+    int nsm = 0;
     {
         // set-up, once per device (and context), with that device current: the
         // host-side name of the array is not a device address, so ask the
@@ -188,16 +235,30 @@ extern "C" int gp_eval_small_noalloc(const uint8_t* d_ops, size_t ops_bytes, con
             void* p = nullptr;
             // (creates the device's context if it does not exist yet)
             if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess) return GP_ECUDA;
+            if (cudaFuncSetAttribute(k_eval_small_noalloc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)NaLayout<1>::total) != cudaSuccess ||
+                cudaFuncSetAttribute(k_eval_small_noalloc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)NaLayout<2>::total) != cudaSuccess ||
+                cudaDeviceGetAttribute(&g_na_nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+                return GP_ECUDA;
             g_na_ptr[dev] = static_cast<float*>(p);
             g_na_ctx[dev] = current_context();
         }
         scratch = g_na_ptr[dev];
+        nsm = g_na_nsm[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the work counter and the status word start at zero on every call
+    // the work counter, the status word and the stacks in use start at zero on every call
     if (cudaMemsetAsync(scratch + NA_OVF_FLOATS, 0, 64 * sizeof(float), st) != cudaSuccess) return GP_ECUDA;
     NaArgs a{d_ops, ops_bytes, d_off, n_trees, d_x, d_t, d_consts, n_cases, d_values, d_fitness, scratch};
-    k_eval_small_noalloc<<<NA_CTAS, NA_WARPS * 32, 0, st>>>(a);
+    // (four cases per lane would halve the window: most larger trees would then queue for an overflow stack, 970 us
+    // instead of 133 us for 3,000 trees x 100 cases)
+    const int K = n_cases <= 32 ? 1 : 2;
+    const uint32_t ncb = (n_cases + 32 * K - 1) / (32 * K);
+    const uint32_t by_cta = (ncb > 1 && n_trees <= (uint32_t)nsm) ? 1u : 0u;
+    const uint32_t grid = n_trees < (uint32_t)nsm ? n_trees : (uint32_t)nsm;
+    if (K == 1) k_eval_small_noalloc<1><<<grid, NA_WARPS * 32, NaLayout<1>::total, st>>>(a, by_cta);
+    else k_eval_small_noalloc<2><<<grid, NA_WARPS * 32, NaLayout<2>::total, st>>>(a, by_cta);
     if (cudaGetLastError() != cudaSuccess) return GP_ECUDA;
     uint32_t flags = 0;
     if (cudaMemcpyAsync(&flags, scratch + NA_OVF_FLOATS + 1, sizeof flags, cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -205,6 +266,7 @@ extern "C" int gp_eval_small_noalloc(const uint8_t* d_ops, size_t ops_bytes, con
     if (cudaStreamSynchronize(st) != cudaSuccess) return GP_ECUDA;
     if (status_out) *status_out = flags;
     if (flags & 1u) return GP_ECAPACITY;
+    if (flags & 4u) return GP_ETIMEOUT;
     if (flags & 2u) return GP_EINVAL;
     return GP_OK;
 }
