@@ -538,7 +538,8 @@ __device__ __forceinline__ bool fx_run(LD ld, uint32_t s, uint32_t e, uint32_t w
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = 0.f;
     for (;;) {
-        if (stop && *stop) { *aborted = true; return true; }
+        // (one decision for the warp: what follows needs all of its lanes)
+        if (stop && __any_sync(FULL, *stop != 0u)) { *aborted = true; return true; }
         const uint32_t fl = fx_funcs(wl);
         const uint32_t wn = fx_word(ld, base - 2 * FX_CHUNK + 4 * lane, s, e);     // in flight during this chunk
         const FxChunk ch = fx_decode<V, false, FxTable<K, V>::row>(cy, fl, base, s, e, c.code, c.lt, 0u);

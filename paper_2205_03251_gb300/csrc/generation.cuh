@@ -2,7 +2,7 @@
 // incremental evaluation of the children with failed disruption
 // propagation (Sec. 5, Sec. 6.2, Sec. 6.3, Fig. 1-3).
 #pragma once
-#include "interp.cuh"
+#include "fused.cuh"
 #include "structure.cuh"
 #include "mlp.cuh"
 
@@ -128,14 +128,46 @@ __device__ __forceinline__ int32_t find_exact(const uint32_t* e_pos, uint32_t lo
     }
     return -1;
 }
-// Last entry with position < x in [lo, hi), or -1.
-__device__ __forceinline__ int32_t find_last_lt(const uint32_t* e_pos, uint32_t lo, uint32_t hi, uint32_t x) {
-    uint32_t a = lo, b = hi;            // first index with pos >= x
-    while (a < b) {
-        uint32_t mid = (a + b) >> 1;
-        if (e_pos[mid] < x) a = mid + 1; else b = mid;
+// Warp-collective: first index in [lo, hi) of the sorted array a with
+// a[i] >= x (hi if none), by 32-way splitting (two rounds for 1,000 entries).
+__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* a, uint32_t lo, uint32_t hi, uint32_t x) {
+    const uint32_t lane = (uint32_t)lane_id();
+    while (hi - lo > 32) {
+        const uint32_t step = (hi - lo + 31) / 32;
+        const uint32_t last = min(lo + (lane + 1) * step, hi) - 1;     // last index of this lane's segment
+        const uint32_t m = __ballot_sync(FULL, a[last] >= x);
+        if (!m) return hi;
+        const uint32_t f = (uint32_t)__ffs(m) - 1;                      // first segment ending at >= x
+        const uint32_t nlo = lo + f * step;
+        hi = min(nlo + step, hi);
+        lo = nlo;
     }
-    return (a > lo) ? (int32_t)(a - 1) : -1;
+    const uint32_t i = lo + lane;
+    const uint32_t m = __ballot_sync(FULL, i < hi && a[i] >= x);
+    return m ? lo + (uint32_t)__ffs(m) - 1 : hi;
+}
+
+// Warp-collective: the deepest cached node that holds position c, from the
+// last entry e before c down (-1: none): the entries before c in a window of
+// 32 are tested at once, and where none of them holds c the parent of the
+// lowest is the next that can (entries between the two lie inside that parent
+// and end before the lowest).  One round trip to memory for 32 entries; parent
+// links alone cost one for each node of the path to the anchor, which in a
+// uniform random tree is long.
+__device__ __forceinline__ int32_t warp_anchor(const CacheView& par, uint32_t me0, int32_t e, uint32_t c) {
+    const int32_t lane = lane_id();
+    uint32_t guard = 0;
+    while (e >= (int32_t)me0 && guard++ < (1u << 24)) {
+        const int32_t x = e - lane;
+        const bool in = x >= (int32_t)me0;
+        const uint32_t end = in ? par.e_end[x] : 0u;
+        const int32_t up = in ? par.e_par[x] : -1;
+        const uint32_t hit = __ballot_sync(FULL, in && end > c);
+        if (hit) return e - (__ffs(hit) - 1);
+        if (e - 31 <= (int32_t)me0) return -1;
+        e = __shfl_sync(FULL, up, 31);
+    }
+    return -1;
 }
 
 // 16 bytes starting at any address (two aligned loads and a funnel shift);
@@ -169,8 +201,8 @@ __device__ __forceinline__ uint4 load16u(const uint8_t* p) {
 __device__ uint32_t warp_subtree_size_at(const CacheView& par, uint32_t t, const uint8_t* ops, uint32_t n,
                                          uint32_t x) {
     const int lane = lane_id();
-    const int32_t e = find_exact(par.e_pos, par.e_off[t], par.e_off[t + 1], x);
-    if (e >= 0) return par.e_end[e] - x;
+    const uint32_t hi = par.e_off[t + 1], j = warp_lower_bound(par.e_pos, par.e_off[t], hi, x);
+    if (j < hi && par.e_pos[j] == x) return par.e_end[j] - x;
     int bal = 1;                                      // nodes still needed at the window start
     for (uint32_t w0 = x; w0 < n; w0 += 512) {
         const uint32_t p0 = w0 + 16u * lane;
@@ -961,18 +993,20 @@ __device__ __forceinline__ void load_blk(const float* row, uint32_t cb, float (&
 // of a batch, the running value vectors of the child and of the mother,
 // the siblings' vectors of a batch, a few broadcast words, then per warp an
 // interpreter stack and two staging buffers.
-struct LevelDesc {
-    uint32_t p, pend, ss, se;   // ancestor, its end in the child, sibling range [ss, se)
-    int32_t pent, sib;          // mother cache entry of p (-1: small) and of the sibling (-1: interpret)
-    uint32_t flags;             // op | left << 8 | child-cached << 9 | bad range << 10 | missing sibling << 11
+struct __align__(16) LevelDesc {
+    uint32_t ss, se;            // sibling range in the child
+    uint32_t p, pend;           // ancestor, its end in the child
+    int32_t pent;               // mother cache entry of p (-1: small)
+    uint32_t sslot;             // value slot of the sibling in the mother's cache (LD_SLOT)
+    uint32_t flags;             // op | LD_* flags | the sibling's opcode << 24 (LD_LEAF)
     int32_t k;                  // ancestor index along the path
-    uint32_t pslot, sslot;      // value slots of pent and sib in the mother's cache
-    uint32_t pad0, pad1;
 };
-#define LD_LEFT (1u << 8)
-#define LD_CACHED (1u << 9)
-#define LD_BAD (1u << 10)
-#define LD_NOSIB (1u << 11)
+#define LD_LEFT (1u << 8)       // the path comes from the left child
+#define LD_CACHED (1u << 9)     // the child caches the ancestor
+#define LD_BAD (1u << 10)       // bad range
+#define LD_NOSIB (1u << 11)     // large sibling without a cache entry
+#define LD_SLOT (1u << 12)      // the sibling's values are in a slot
+#define LD_LEAF (1u << 13)      // the sibling is a leaf
 
 #define WALK_RING 32           // most levels a walk team keeps in flight (descriptors and sibling values)
 #define WALK_SPIN (1u << 22)   // default bound on the polls of one wait inside a walk team (DevPop::wait_polls)
@@ -980,13 +1014,13 @@ struct LevelDesc {
 // levels in flight: fewer when value vectors are long
 __host__ __device__ inline uint32_t walk_ring(uint32_t Cpad) { return Cpad <= 128 ? 32u : Cpad <= 256 ? 8u : 4u; }
 
+// (tab: bytes of the interpreter's leaf table, first so that its addresses fit 16 bits)
 template <int K>
 struct TeamLayout {
-    uint32_t kc, anc, ancg, lvl, desc, nv, ov, sv, mv, cur, sc, warp0, warp_bytes, total;
-    __host__ __device__ TeamLayout(int W, uint32_t Cpad, uint32_t nw) {
+    uint32_t anc, ancg, lvl, desc, nv, ov, sv, sc, warp0, warp_bytes, total;
+    __host__ __device__ TeamLayout(int W, uint32_t Cpad, uint32_t nw, uint32_t tab) {
         const uint32_t ring = walk_ring(Cpad);
-        uint32_t o = 0;
-        kc = o;   o += (256 + 6 * 32) * 4;
+        uint32_t o = tab;
         anc = o;  o += WALK_MAXLVL * 4;
         ancg = o; o += WALK_MAXLVL * 4;
         lvl = o;  o += WALK_MAXLVL * 4;
@@ -994,52 +1028,42 @@ struct TeamLayout {
         nv = o;   o += Cpad * 4;
         ov = o;   o += Cpad * 4;
         sv = o;   o += ring * Cpad * 4;
-        mv = o;   o += ring * Cpad * 4;
-        o = (o + 15u) & ~15u;
-        cur = o;  o += 16;                                                  // evaluators' next item
         sc = o;   o += (16 + 2 * WALK_RING) * 4;
         o = (o + 15u) & ~15u;
         warp0 = o;
-        warp_bytes = (uint32_t)W * 32 * K * 4 + 2 * STAGE_BYTES;
+        warp_bytes = (uint32_t)W * 32 * K * 4 + FX_CODE_BYTES;
         total = o + nw * warp_bytes;
     }
 };
 
-// left/right combination keeping the operand order of the node
+// Evaluate bytes [s, e) of `src` (a run below the threshold; src on a 4-byte
+// boundary); false when `stop` ended it.  Out of line: the walk calls it from
+// several places, and with a copy of the interpreter in each of them the
+// combining warp spent most of its time fetching instructions (2.5 us a level).
 template <int K, int V>
-__device__ __forceinline__ void combine(uint32_t op, bool path_left, float (&v)[K], const float (&sib)[K]) {
-    if (path_left) apply_vec<K, V>(op, v, sib);
-    else {
-        float t[K];
+__device__ __noinline__ bool eval_run(const uint8_t* src, uint32_t s, uint32_t e, const FxCtx<K>& c, float (&out)[K],
+                                      uint32_t* status, const volatile uint32_t* stop) {
+    const FxCtx<K> ctx = c;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(src);
+    auto ld = [&](uint32_t q) { return __ldg(words + (q >> 2)); };
+    uint32_t w0, w1;
+    fx_first(ld, s, e, w0, w1);
+    bool aborted = false;
+    float v[K];
+    if (!fx_run<K, V>(ld, s, e, w0, w1, ctx, v, FxHave(), stop, &aborted) && lane_id() == 0) set_status(status, ST_STACK);
 #pragma unroll
-        for (int k = 0; k < K; ++k) t[k] = sib[k];
-        apply_vec<K, V>(op, t, v);
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = t[k];
-    }
+    for (int k = 0; k < K; ++k) out[k] = v[k];
+    return !aborted;
 }
 
-// Evaluate bytes [s, e) of `src` (a small run: e - (s & ~15) <= STAGE_BYTES).
-template <int K, int V>
-__device__ __forceinline__ void eval_run(const uint8_t* src, uint32_t s, uint32_t e, uint8_t* stage,
-                                         const Ictx<K>& c, float (&out)[K], uint32_t* status,
-                                         const volatile uint32_t* stop = nullptr, bool* aborted = nullptr) {
-    __syncwarp();
-    stage_issue(stage, src, s, e);
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncwarp();
-    Istate<K> st;
+// 32 bytes at `p` (on a 32-byte boundary): bit i set when byte i is a function.
+__device__ __forceinline__ uint32_t func_bits32(const uint8_t* p) {
+    const uint4 a = __ldg(reinterpret_cast<const uint4*>(p)), b = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t m = 0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) st.acc[k] = 0.f;
-    st.sp = 0;
-    st.ok = true;
-    bool ab = false;
-    interp_staged_lone<K, V>(stage, s, e, st, c, stop, &ab);
-    if (ab) { if (aborted) *aborted = true; return; }
-    if (!st.ok && lane_id() == 0) set_status(status, ST_STACK);
-#pragma unroll
-    for (int k = 0; k < K; ++k) out[k] = st.acc[k];
+    for (int i = 0; i < 8; ++i) m |= (((fx_funcs(w[i]) & 0x08040201u) * 0x01010101u) >> 24) << (4 * i);
+    return m;
 }
 
 // Ancestors of the crossover point c in the child, for one warp: the
@@ -1047,94 +1071,100 @@ __device__ __forceinline__ void eval_run(const uint8_t* src, uint32_t s, uint32_
 // (positions anc[], balance offsets ancg[], nearest first) from a backward
 // balance scan over at most T bytes before c, and the child ends of those
 // levels (lvl[v] = end of the ancestor whose subtree closes at balance v)
-// from a forward scan after the donated subtree.  Returns false on an
-// inconsistency (recorded in the status word).
+// from a forward scan after the donated subtree.  A lane holds 32 positions
+// as a bit mask of functions, read straight from the tree.  Returns false on
+// an inconsistency (recorded in the status word).
 template <int K>
-__device__ bool walk_ancestors(const DevPop& d, const CacheView& par, uint32_t i, const uint8_t* ok_, int32_t tdl,
-                               uint32_t c,
-                               uint32_t s, uint32_t nk, int32_t em, uint32_t me0, uint32_t me1, uint8_t* stB,
-                               uint32_t* anc, int32_t* ancg, uint32_t* lvl, int32_t& A_out, uint32_t& nsmall_out,
-                               int32_t& hneed_out) {
-    const int lane = lane_id();
+__device__ __noinline__ bool walk_ancestors(const DevPop& d, const CacheView& par, uint32_t i, const uint8_t* ok_,
+                                            int32_t tdl, uint32_t c, uint32_t s, uint32_t nk, int32_t em, uint32_t me0,
+                                            uint32_t me1, uint32_t* anc, int32_t* ancg, uint32_t* lvl, int32_t& A_out,
+                                            uint32_t& nsmall_out, int32_t& hneed_out) {
+    const uint32_t lane = (uint32_t)lane_id();
     const uint32_t T = d.T;
     int32_t A = -1;
     uint32_t nsmall = 0;
     if (em >= 0) A = par.e_par[em];
     else {
-        int32_t e = find_last_lt(par.e_pos, me0, me1, c);
-        uint32_t guard = 0;
-        while (e >= 0 && par.e_end[e] <= c && guard++ < (1u << 24)) e = par.e_par[e];
-        A = e;
+        A = warp_anchor(par, me0, (int32_t)warp_lower_bound(par.e_pos, me0, me1, c) - 1, c);
         if (A < 0) { if (lane == 0) set_error(d, ST_STRUCT, 5, i, c, 0); return false; }
         // backward scan of (max(pos(A)+1, c-T+1) .. c-1]: G(j) = sum_{k=j}^{c-1} (arity_k - 1);
         // j is an ancestor of c iff G(j) >= G(m) for every m in (j, c], G(c) = 0
         const uint32_t pA = par.e_pos[A];
         const uint32_t lo = max(pA + 1, (c + 1 > T) ? c + 1 - T : 0u);
         if (lo < c) {
-            __syncwarp();
-            stage_issue(stB, ok_, lo, c);
-            cp_async_commit();
-            cp_async_wait<0>();
-            __syncwarp();
-            const uint32_t a16 = lo & ~15u;
-            // lane l: positions c-1-32l-t, t = 0..31 (nearest first)
-            int sum = 0, mx = -0x40000000;
-            for (int t = 0; t < 32; ++t) {
-                const int64_t j = (int64_t)c - 1 - 32 * lane - t;
-                if (j >= (int64_t)lo) { sum += (stB[j - a16] < 4) ? 1 : -1; mx = max(mx, sum); }
-            }
-            // G offset from the lanes nearer to c, and the maximum G seen before this lane
-            int incl = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int ts = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += ts;
-            }
-            const int base = incl - sum;
-            int pm = (mx > -0x40000000) ? base + mx : -0x40000000;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int tm = __shfl_up_sync(FULL, pm, o);
-                if (lane >= o) pm = max(pm, tm);
-            }
-            int prevmax = __shfl_up_sync(FULL, pm, 1);
-            if (lane == 0) prevmax = 0;            // G(c) = 0
-            prevmax = max(prevmax, 0);
-            uint32_t fmask = 0;
-            int run = prevmax, gsum = base;
-            for (int t = 0; t < 32; ++t) {
-                const int64_t j = (int64_t)c - 1 - 32 * lane - t;
-                if (j >= (int64_t)lo) {
-                    gsum += (stB[j - a16] < 4) ? 1 : -1;
-                    if (gsum >= run) { fmask |= 1u << t; run = gsum; }
+            // lane l: the 32 positions of block B - l, nearest first from its top bit down
+            // (T - 1 <= 1,023 positions touch at most 33 blocks: the farthest, beyond lane 31, in a second round)
+            const int32_t B = (int32_t)((c - 1) / 32);
+            int gin = 0, pmin = 0;              // G before this round, its largest value so far
+#pragma unroll 1
+            for (int32_t rnd = 0; rnd < 2 && 32 * (B - 32 * rnd) + 31 >= (int32_t)lo; ++rnd) {
+                const int32_t blk = B - 32 * rnd - (int32_t)lane;
+                uint32_t valid = 0, F = 0;
+                if (blk >= 0 && 32 * blk + 31 >= (int32_t)lo) {
+                    const uint32_t p0 = 32u * (uint32_t)blk;
+                    valid = 0xFFFFFFFFu;
+                    if (p0 < lo) valid &= 0xFFFFFFFFu << (lo - p0);
+                    if (p0 + 32 > c) valid &= 0xFFFFFFFFu >> (p0 + 32 - c);
+                    F = func_bits32(ok_ + p0) & valid;
                 }
-            }
-            // compact in nearest-first order
-            const uint32_t cnt = __popc(fmask);
-            uint32_t off = cnt;
+                // sum and largest partial sum of the lane's positions, from the top bit down
+                int sum = 0, mx = -64;
+#pragma unroll 1
+                for (int t = 31; t >= 0; --t) {
+                    if (valid >> t & 1u) { sum += (F >> t & 1u) ? 1 : -1; mx = max(mx, sum); }
+                }
+                int incl = sum;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                uint32_t tt = __shfl_up_sync(FULL, off, o);
-                if (lane >= o) off += tt;
-            }
-            off -= cnt;
-            const uint32_t tot = __shfl_sync(FULL, off + cnt, 31);
-            if (tot > WALK_MAXLVL - 2) { if (lane == 0) set_status(d.status, ST_PATH); return false; }
-            gsum = base;
-            uint32_t k = off;
-            for (int t = 0; t < 32; ++t) {
-                const int64_t j = (int64_t)c - 1 - 32 * lane - t;
-                if (j >= (int64_t)lo) {
-                    gsum += (stB[j - a16] < 4) ? 1 : -1;
-                    if (fmask & (1u << t)) {
-                        anc[k] = (uint32_t)j;
-                        // balance offset (>= 0 at an ancestor), operator byte in bits 24..
-                        ancg[k] = (int32_t)((uint32_t)gsum | ((uint32_t)stB[j - a16] << 24));
-                        ++k;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(FULL, incl, o);
+                    if ((int)lane >= o) incl += v;
+                }
+                const int base = gin + incl - sum;
+                int pm = valid ? base + mx : -0x40000000;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(FULL, pm, o);
+                    if ((int)lane >= o) pm = max(pm, v);
+                }
+                int run = __shfl_up_sync(FULL, pm, 1);
+                if (lane == 0) run = pmin;
+                run = max(run, pmin);
+                // the records: positions where G reaches a new largest value or equals it
+                uint32_t rec = 0;
+                int gs = base, gr = run;
+#pragma unroll 1
+                for (int t = 31; t >= 0; --t) {
+                    if (valid >> t & 1u) {
+                        gs += (F >> t & 1u) ? 1 : -1;
+                        if (gs >= gr) { rec |= 1u << t; gr = gs; }
                     }
                 }
+                const uint32_t cnt = __popc(rec);
+                uint32_t off = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(FULL, off, o);
+                    if ((int)lane >= o) off += v;
+                }
+                const uint32_t tot = __shfl_sync(FULL, off, 31);
+                off += nsmall - cnt;
+                if (nsmall + tot > WALK_MAXLVL - 2) { if (lane == 0) set_status(d.status, ST_PATH); return false; }
+                while (rec) {
+                    const int t = 31 - __clz(rec);
+                    rec &= ~(1u << t);
+                    const uint32_t j = 32u * (uint32_t)blk + (uint32_t)t;
+                    // G there: the positions from t up
+                    const uint32_t up = 0xFFFFFFFFu << t;
+                    const int g = base + 2 * __popc(F & up) - __popc(valid & up);
+                    anc[off] = j;
+                    // balance offset (>= 0 at an ancestor), operator byte in bits 24..
+                    ancg[off] = (int32_t)((uint32_t)g | ((uint32_t)ok_[j] << 24));
+                    ++off;
+                }
+                nsmall += tot;
+                gin += __shfl_sync(FULL, incl, 31);
+                pmin = max(pmin, __shfl_sync(FULL, pm, 31));
             }
-            nsmall = tot;
             __syncwarp();
         }
     }
@@ -1146,44 +1176,57 @@ __device__ bool walk_ancestors(const DevPop& d, const CacheView& par, uint32_t i
     int32_t hneed = -1;
     if (nsmall) {
         const uint32_t f0 = c + s;
-        const uint32_t f1 = f0 + T;
         // sentinel 0 for levels the scan does not reach: their sibling ranges then fail the
         // size check of the walk instead of reading a stale end
         for (uint32_t v = lane; v <= maxv; v += 32) lvl[v] = 0;
         __syncwarp();
-        // child positions q >= c + s are bytes q - tdl of ok_
-        const uint32_t lim = min(f1, (nk + 15u) & ~15u);
-        if (f0 < lim) { stage_issue(stB, ok_, f0 - tdl, lim - tdl); }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncwarp();
-        const uint32_t a16 = ((f0 - tdl) & ~15u) + tdl;
         if (lane == 0) lvl[1] = f0;
-        int sum = 0, mx = 0;
-        // lane l: positions f0 + 32l + t
-        for (int t = 0; t < 32; ++t) {
-            const uint32_t q = f0 + 32 * lane + t;
-            const int w = (q < nk && stB[q - a16] < 4) ? -1 : 1;
-            sum += w;
-            mx = max(mx, sum);
-        }
-        int incl = sum;
+        // child positions q >= c + s are bytes q - tdl of ok_: lane l the 32 bytes of block (f0 - tdl) / 32 + l, at most
+        // T of them from f0 on (33 blocks, as above); positions past the child's end count as leaves, +1 each
+        const uint32_t g0 = f0 - (uint32_t)tdl, gend = nk - (uint32_t)tdl;      // bytes [g0, gend) of ok_
+        int bin = 1;                           // balance before this round
+        int best = 1;                          // largest balance so far
+#pragma unroll 1
+        for (uint32_t rnd = 0; rnd < 2; ++rnd) {
+            const uint32_t p0 = 32u * (g0 / 32 + 32 * rnd + lane);
+            uint32_t valid = 0, F = 0;
+            if (p0 + 32 > g0 && p0 < g0 + T) {
+                valid = 0xFFFFFFFFu;
+                if (p0 < g0) valid &= 0xFFFFFFFFu << (g0 - p0);
+                if (p0 + 32 > g0 + T) valid &= 0xFFFFFFFFu >> (p0 + 32 - (g0 + T));
+                if (p0 < gend) F = func_bits32(ok_ + p0) & valid;
+                if (p0 < gend && p0 + 32 > gend) F &= 0xFFFFFFFFu >> (p0 + 32 - gend);
+            }
+            int sum = 0, mx = -64;
+#pragma unroll 1
+            for (int t = 0; t < 32; ++t) {
+                if (valid >> t & 1u) { sum += (F >> t & 1u) ? -1 : 1; mx = max(mx, sum); }
+            }
+            int incl = sum;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { int ts = __shfl_up_sync(FULL, incl, o); if (lane >= o) incl += ts; }
-        const int base = 1 + incl - sum;          // balance before the lane's first position
-        int lmax = base + mx;                      // max after-balance in the lane (or base)
-        lmax = max(lmax, base);
-        int pm = lmax;
+            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(FULL, incl, o); if ((int)lane >= o) incl += v; }
+            const int base = bin + incl - sum;
+            int pm = valid ? base + mx : -0x40000000;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { int tm = __shfl_up_sync(FULL, pm, o); if (lane >= o) pm = max(pm, tm); }
-        int prev = __shfl_up_sync(FULL, pm, 1);
-        if (lane == 0) prev = 1;
-        prev = max(prev, base);
-        int bal = base;
-        for (int t = 0; t < 32; ++t) {
-            const uint32_t q = f0 + 32 * lane + t;
-            bal += (q < nk && stB[q - a16] < 4) ? -1 : 1;
-            if (bal > prev) { if ((uint32_t)bal < WALK_MAXLVL) lvl[bal] = q + 1; prev = bal; }
+            for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(FULL, pm, o); if ((int)lane >= o) pm = max(pm, v); }
+            int prev = __shfl_up_sync(FULL, pm, 1);
+            if (lane == 0) prev = best;
+            prev = max(prev, best);
+            int bal = base;
+#pragma unroll 1
+            for (int t = 0; t < 32; ++t) {
+                if (valid >> t & 1u) {
+                    bal += (F >> t & 1u) ? -1 : 1;
+                    if (bal > prev) {
+                        if ((uint32_t)bal < WALK_MAXLVL) lvl[bal] = p0 + t + 1 + (uint32_t)tdl;
+                        prev = bal;
+                    }
+                }
+            }
+            bin += __shfl_sync(FULL, incl, 31);
+            best = max(best, __shfl_sync(FULL, pm, 31));
+            // (uniform) the second round only when the first did not cover T bytes or reach the last level
+            if (best >= (int)maxv) break;
         }
         __syncwarp();
         // highest small ancestor that the child caches (needs a value even above the stop)
@@ -1192,8 +1235,7 @@ __device__ bool walk_ancestors(const DevPop& d, const CacheView& par, uint32_t i
             const uint32_t pe = lvl[(ancg[k] & 0xFFFFFF) + 1];
             if (pe - p >= T) hneed = max(hneed, (int32_t)k);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) hneed = max(hneed, __shfl_xor_sync(FULL, hneed, o));
+        hneed = __reduce_max_sync(FULL, hneed);
     }
     A_out = A;
     nsmall_out = nsmall;
@@ -1260,85 +1302,120 @@ __device__ __forceinline__ void dis_store(const GenBufs& g, uint32_t i, uint32_t
 // values of nodes that are cached in the child are recorded for the
 // child's cache; above the stop only child-cached nodes that the mother
 // does not cache need computing.
-// Builder of the walk's level descriptors (one lane): the ancestors of the
-// crossover point from the nearest up -- the small ones from the backward
-// balance scan (anc, ancg, lvl), then the mother's cached ancestors through
-// their parent links -- each with its sibling's range in the child and, for
-// a large sibling, its cache entry.  `stopped` ends the building above the
-// stop except for small ancestors that the child caches (they need values).
-
+// Builder of the walk's level descriptors (warp 0, all lanes): up to 32
+// levels at a time, the ancestors of the crossover point from the nearest up
+// -- the small ones from the backward balance scan (anc, ancg, lvl), then the
+// mother's cached ancestors -- each with its sibling's range in the child
+// and, for a large sibling, its value slot.  Cached ancestors come from the
+// 32 entries up to the nearest one: an entry there is an ancestor when its
+// subtree holds the crossover point (entries that are not belong to siblings
+// on the left; on a chain of nodes with one large child there are none).  So
+// 32 levels cost two round trips to memory, where following the parent links
+// cost two for each level.
 struct WalkBuilder {
-    uint32_t bq, bqend, bk;
-    int32_t bpe;
-    bool btop;
+    uint32_t bq, bqend, bk;    // the path's child at the next level: position, end; levels built
+    int32_t bpe;               // next cached ancestor's entry, or -1
+    bool btop;                 // nothing left to build
 };
 
 struct WalkCtx {
     const uint8_t* ok_;        // child bytes before the crossover point (the mother's in fitness-first order)
-    uint32_t nsmall, nk, s, r, T;
+    uint32_t nsmall, nk, s, r, c, T, me0;
+    int32_t tdl;               // child position x >= c + s is byte x - tdl of ok_
     int32_t A, hneed;
     const uint32_t* anc;
     const int32_t* ancg;
     const uint32_t* lvl;
 };
 
-// Build the next level into D; false (and btop set) when there is none.
-// The walk's critical path on long paths runs through this builder, one
-// dependent chain of cache-link loads per level: every field of a cached
-// ancestor's entry is loaded at once (one round trip), then its operator
-// byte and its large sibling's slot (a second one); a small ancestor's
-// operator byte was kept by the backward scan (bits 24.. of ancg).
-__device__ __forceinline__ bool build_level(const CacheView& par, const WalkCtx& w, WalkBuilder& b, bool stopped,
-                                            LevelDesc& D) {
-    if (b.btop) return false;
-    uint32_t p, pend, op;
-    int32_t pent, c0 = -1, c1 = -1, nextp = -1;
-    uint32_t pslot = 0;
+// Build at most `room` levels (1..32) into the ring from level nb on; returns
+// how many.  Once the walk has stopped only small ancestors that the child
+// caches are needed.
+__device__ __forceinline__ uint32_t build_levels(const CacheView& par, const WalkCtx& w, WalkBuilder& b, bool stopped,
+                                                 LevelDesc* desc, volatile uint32_t* dtag, uint32_t ring, uint32_t nb,
+                                                 uint32_t room) {
+    const uint32_t lane = (uint32_t)lane_id();
+    if (b.btop) return 0u;
+    bool in;                                   // this lane has a level
+    uint32_t rank, p = 0, pend = 0, op = 0;
+    int32_t pent = -1, c0 = -1, c1 = -1, up = -1;
+    uint32_t mask;
     if (b.bk < w.nsmall) {
-        const int32_t gk = w.ancg[b.bk];
-        p = w.anc[b.bk];
-        pend = w.lvl[(gk & 0xFFFFFF) + 1];
-        op = (uint32_t)gk >> 24;
-        pent = -1;
+        uint32_t cnt = min(min(32u, room), w.nsmall - b.bk);
+        if (stopped) cnt = min(cnt, (uint32_t)max(0, w.hneed + 1 - (int32_t)b.bk));
+        if (cnt == 0) { b.btop = true; return 0u; }
+        in = lane < cnt;
+        rank = lane;
+        mask = __ballot_sync(FULL, in);
+        if (in) {
+            const int32_t gk = w.ancg[b.bk + lane];
+            p = w.anc[b.bk + lane];
+            pend = w.lvl[(gk & 0xFFFFFF) + 1];
+            op = (uint32_t)gk >> 24;
+        }
     } else {
-        pent = (b.bk == w.nsmall) ? w.A : b.bpe;
-        if (pent < 0) { b.btop = true; return false; }                  // above the root
-        p = __ldg(par.e_pos + pent);
-        const uint32_t e = __ldg(par.e_end + pent);
-        c0 = __ldg(par.e_c0 + pent);
-        c1 = __ldg(par.e_c1 + pent);
-        pslot = __ldg(par.e_slot + pent);
-        nextp = __ldg(par.e_par + pent);
-        pend = (uint32_t)((int64_t)e + ((int64_t)w.s - (int64_t)w.r));
-        op = 0xFFFFFFFFu;
+        const int32_t top = (b.bk == w.nsmall) ? w.A : b.bpe;
+        if (top < 0 || stopped) { b.btop = true; return 0u; }
+        const int32_t idx = top - (int32_t)lane;
+        in = idx >= (int32_t)w.me0;
+        if (in) {
+            p = __ldg(par.e_pos + idx);
+            const uint32_t e = __ldg(par.e_end + idx);
+            c0 = __ldg(par.e_c0 + idx);
+            c1 = __ldg(par.e_c1 + idx);
+            up = __ldg(par.e_par + idx);
+            pend = (uint32_t)((int64_t)e + ((int64_t)w.s - (int64_t)w.r));
+            in = e > w.c && p < w.c;
+            pent = idx;
+        }
+        mask = __ballot_sync(FULL, in);
+        rank = __popc(mask & ((1u << lane) - 1u));
+        in = in && rank < room;
+        mask = __ballot_sync(FULL, in);
+        if (in) op = w.ok_[p];
     }
-    // above the stop only small ancestors that the child caches need values
-    if (stopped && (pent >= 0 || (int32_t)b.bk > w.hneed)) { b.btop = true; return false; }
-    const bool left = (b.bq == p + 1);
-    const uint32_t ss = left ? b.bqend : p + 1;
-    const uint32_t se = left ? pend : b.bq;
-    int32_t sib = -1;
-    uint32_t bad = 0;
-    if (se <= ss || se > w.nk) bad = LD_BAD;
-    else if (se - ss >= w.T) {
-        sib = (pent < 0) ? -1 : (left ? c1 : c0);
-        if (sib < 0) bad = LD_NOSIB;
+    const uint32_t n = __popc(mask);
+    if (n == 0) { b.btop = true; return 0u; }          // (an inconsistent cache: its links lead nowhere)
+    // the path's child at this level: the lane of the level below
+    const uint32_t below = mask & ((1u << lane) - 1u);
+    const int from = below ? 31 - __clz(below) : (int)lane;
+    uint32_t q = __shfl_sync(FULL, p, from), qend = __shfl_sync(FULL, pend, from);
+    if (!below) { q = b.bq; qend = b.bqend; }
+    const bool left = q == p + 1;
+    const uint32_t ss = left ? qend : p + 1, se = left ? pend : q;
+    uint32_t flg = 0, sslot = 0;
+    if (in) {
+        flg = op | (left ? LD_LEFT : 0u) | ((p == 0 || pend - p >= w.T) ? LD_CACHED : 0u);
+        if (se <= ss || se > w.nk) flg |= LD_BAD;
+        else if (se - ss >= w.T) {
+            const int32_t sib = (pent < 0) ? -1 : (left ? c1 : c0);
+            if (sib < 0) flg |= LD_NOSIB;
+            else { flg |= LD_SLOT; sslot = __ldg(par.e_slot + sib); }
+        } else if (se - ss == 1) {
+            flg |= LD_LEAF | ((uint32_t)w.ok_[ss - (left ? w.tdl : 0)] << 24);
+        }
     }
-    if (op == 0xFFFFFFFFu) op = w.ok_[p];
-    const uint32_t sslot = (sib >= 0) ? __ldg(par.e_slot + sib) : 0u;
-    const uint32_t flg = op | (left ? LD_LEFT : 0u) | ((p == 0 || pend - p >= w.T) ? LD_CACHED : 0u) | bad;
-    D.p = p; D.pend = pend; D.ss = ss; D.se = se; D.pent = pent; D.sib = sib; D.flags = flg;
-    D.k = (int32_t)b.bk;
-    D.pslot = pslot;
-    D.sslot = sslot;
-    D.pad0 = 0u; D.pad1 = 0u;
-    if (bad) { b.btop = true; return true; }
-    b.bq = p;
-    b.bqend = pend;
-    if (b.bk >= w.nsmall) b.bpe = nextp;
-    ++b.bk;
-    if (p == 0) b.btop = true;
-    return true;
+    // up to and including the first level that cannot be combined
+    const uint32_t bad = __ballot_sync(FULL, in && (flg & (LD_BAD | LD_NOSIB)));
+    const uint32_t root = __ballot_sync(FULL, in && p == 0);
+    const uint32_t end = bad | root;
+    const uint32_t nn = end ? __popc(mask & (2u * (1u << (__ffs(end) - 1)) - 1u)) : n;
+    const uint32_t slot = (nb + rank) % ring;
+    if (in && rank < nn) {
+        LevelDesc& D = desc[slot];
+        D.ss = ss; D.se = se; D.p = p; D.pend = pend; D.pent = pent; D.sslot = sslot; D.flags = flg;
+        D.k = (int32_t)(b.bk + rank);
+    }
+    __threadfence_block();
+    __syncwarp();
+    if (in && rank < nn) dtag[slot] = (nb + rank + 1) | ((flg & LD_LEAF) ? 0x80000000u : 0u);
+    const int last = 31 - __clz(mask);
+    b.bq = __shfl_sync(FULL, p, last);
+    b.bqend = __shfl_sync(FULL, pend, last);
+    b.bpe = __shfl_sync(FULL, up, last);
+    b.bk += nn;
+    if (end) b.btop = true;
+    return nn;
 }
 
 // The children one launch walks: entries [q_lo, q_hi) of the work order,
@@ -1348,14 +1425,22 @@ struct WalkRange {
     uint32_t q_lo, q_hi, qctr, ovf_base;
 };
 
+// Bound by latency: on 4,096 uneven trees a walk of 58 levels with 1,600
+// interpreted nodes takes a team about 200 us, a third of a warp's cycles
+// waiting for instructions (one warp of a team combines, the others run the
+// interpreter).  Two forms: MAXT 128 keeps 5 teams of 4 warps on an SM (96
+// registers, some spilled) for populations whose children queue for teams;
+// MAXT 512 keeps its registers (4 teams of 4 warps) for populations whose
+// longest walk counts, and for larger teams.  4,096 uneven trees 3.4 -> 1.5 ms
+// (1.65 with the second form), 500 grafted trees of 1e6 nodes 0.30 -> 0.17 ms
+// (0.19 with the first).
 template <int K, int V, int MAXT>
-__global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, CacheView par, uint32_t nw,
+__global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, GenBufs g, CacheView par, uint32_t nw,
                                                            WalkRange wr) {
     if (halted(d)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t Cpad = d.Cpad, Cn = d.C, ncb = d.ncb, T = d.T;
-    const TeamLayout<K> L((int)d.W, Cpad, nw);
-    float* kc = reinterpret_cast<float*>(smem_raw + L.kc);
+    const TeamLayout<K> L((int)d.W, Cpad, nw, FxTable<K, V>::bytes(ncb));
     uint32_t* anc = reinterpret_cast<uint32_t*>(smem_raw + L.anc);
     int32_t* ancg = reinterpret_cast<int32_t*>(smem_raw + L.ancg);
     uint32_t* lvl = reinterpret_cast<uint32_t*>(smem_raw + L.lvl);
@@ -1363,30 +1448,28 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
     float* nvs = reinterpret_cast<float*>(smem_raw + L.nv);
     float* ovs = reinterpret_cast<float*>(smem_raw + L.ov);
     float* svs = reinterpret_cast<float*>(smem_raw + L.sv);
-    float* mvs = reinterpret_cast<float*>(smem_raw + L.mv);
     volatile uint32_t* sc = reinterpret_cast<volatile uint32_t*>(smem_raw + L.sc);
     const int lane = lane_id();
     const uint32_t warp = threadIdx.x >> 5, tid = threadIdx.x;
-    fill_kc(kc, d.consts);
-    fill_kb(kc + 256);
+    FxTable<K, V>::fill(reinterpret_cast<float*>(smem_raw), d.consts, ncb);
     __syncthreads();
-    unsigned char* wb = smem_raw + L.warp0 + warp * L.warp_bytes;
-    Ictx<K> ic;
-    ic.s = reinterpret_cast<float*>(wb);
-    ic.W = (int)d.W;
-    ic.maxd = (int)d.maxdepth;
-    ic.kc = kc;
-    ic.kb = kc + 256;
-    ic.g = d.ovf + (size_t)(wr.ovf_base + blockIdx.x * nw + warp) * (d.maxdepth - d.W) * 32 * K;
-    uint8_t* stA = wb + (size_t)d.W * 32 * K * 4;
-    uint8_t* stB = stA + STAGE_BYTES;
-    volatile uint32_t* dtag = sc + 16;                 // [WALK_RING] level + 1 whose descriptor is in the slot
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    FxCtx<K> ic;
+    ic.stack = sm + L.warp0 + warp * L.warp_bytes + lane * K * 4;
+    ic.code = sm + L.warp0 + warp * L.warp_bytes + d.W * 32 * K * 4;
+    ic.lo = lane * K * 4;
+    ic.W = d.W;
+    ic.maxd = d.maxdepth;
+    ic.g = d.ovf + (size_t)(wr.ovf_base + blockIdx.x * nw + warp) * d.maxdepth * 32 * K;
+    volatile uint32_t* dtag = sc + 16;                 // [WALK_RING] level + 1 whose descriptor is in the slot (bit 31: leaf sibling)
     volatile uint32_t* vcnt = sc + 16 + WALK_RING;     // [WALK_RING] case blocks of the slot's sibling done
-    unsigned long long* cur = reinterpret_cast<unsigned long long*>(smem_raw + L.cur);   // level << 32 | case block
     const uint32_t nev = nw - 1;                       // sibling evaluators (warps 1..nw-1)
     const uint32_t ring = walk_ring(Cpad);
-    const uint32_t ahead = ring;                       // levels built ahead of the combination
-    unsigned long long st_interp = 0, st_levels = 0, st_stopped = 0, st_pathops = 0;
+    uint32_t st_interp = 0, st_levels = 0, st_stopped = 0, st_pathops = 0;
+    auto cases = [&](uint32_t cb) {
+        load_cases<K>(d, cb, ic.x);
+        ic.lt = FxTable<K, V>::at(sm, cb);
+    };
 
     for (;;) {
         if (tid == 0) sc[0] = atomicAdd(&d.q[wr.qctr], 1u);
@@ -1429,11 +1512,13 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
         // ---- level 0: donated subtree vs removed subtree
         int32_t ef = -1, em = -1;
         if (s >= T || dd == 0) {
-            ef = find_exact(par.e_pos, fe0, fe1, dd);
+            const uint32_t j = warp_lower_bound(par.e_pos, fe0, fe1, dd);
+            if (j < fe1 && par.e_pos[j] == dd) ef = (int32_t)j;
             if (ef < 0) { if (tid == 0) set_error(d, ST_STRUCT, 3, i, dd, s); continue; }
         }
         if (r >= T || c == 0) {
-            em = find_exact(par.e_pos, me0, me1, c);
+            const uint32_t j = warp_lower_bound(par.e_pos, me0, me1, c);
+            if (j < me1 && par.e_pos[j] == c) em = (int32_t)j;
             if (em < 0) { if (tid == 0) set_error(d, ST_STRUCT, 4, i, c, r); continue; }
         }
         // the donated subtree becomes the child's root (always cached) but the
@@ -1454,26 +1539,21 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
         // ancestors and builds the first levels; warp 0 compares level 0 just
         // before it combines level 1.  A team of one does them in turn.
         if (tid < WALK_RING) { dtag[tid] = 0u; vcnt[tid] = 0u; }
-        if (tid == 0) { *cur = 0ull; sc[8] = 0u; sc[6] = 0u; sc[4] = 0u; }
+        if (tid == 0) { sc[5] = 0u; sc[8] = 0u; sc[6] = 0u; sc[4] = 0u; }
         __syncthreads();
         auto level0 = [&](uint32_t first, uint32_t step) {
             for (uint32_t it = first; it < 2 * ncb; it += step) {
                 const uint32_t which = it & 1u, cb = it >> 1;
-                load_cases<K>(d, cb, ic.xv);
+                const int32_t ent = which == 0 ? ef : em;
                 float v[K];
-                if (which == 0) {
-                    if (ef >= 0) load_vec<K>(par.slots, Cpad, par.e_slot[ef], v, cb);
-                    else {
-                        if (virt) eval_run<K, V>(d.arena + (size_t)g.pbuf[f] * d.cap, dd, dd + s, stA, ic, v, d.status);
-                        else eval_run<K, V>(ok_, c, c + s, stA, ic, v, d.status);
-                        if (cb == 0) st_interp += s;
-                    }
-                } else {
-                    if (em >= 0) load_vec<K>(par.slots, Cpad, par.e_slot[em], v, cb);
-                    else {
-                        eval_run<K, V>(g.stash + g.stash_off[i], 0, r, stA, ic, v, d.status);
-                        if (cb == 0) st_interp += r;
-                    }
+                if (ent >= 0) load_vec<K>(par.slots, Cpad, par.e_slot[ent], v, cb);
+                else {
+                    // the donated subtree in the father (or in the built child), the removed one in the stash
+                    const uint8_t* src = which ? g.stash + g.stash_off[i] : virt ? d.arena + (size_t)g.pbuf[f] * d.cap : ok_;
+                    const uint32_t from = which ? 0u : virt ? dd : c, len = which ? r : s;
+                    cases(cb);
+                    eval_run<K, V>(src, from, from + len, ic, v, d.status, nullptr);
+                    if (cb == 0) st_interp += len;
                 }
                 store_blk<K>(which == 0 ? nvs : ovs, cb, v);
             }
@@ -1494,27 +1574,30 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
             // ---- ancestors
             int32_t A = -1, hneed = -1;
             uint32_t nsmall = 0;
-            const bool anc_ok = walk_ancestors<K>(d, par, i, ok_, tdl, c, s, nk, em, me0, me1, stB, anc, ancg, lvl, A,
+            const bool anc_ok = walk_ancestors<K>(d, par, i, ok_, tdl, c, s, nk, em, me0, me1, anc, ancg, lvl, A,
                                                   nsmall, hneed);
+            // the running values of the child and the mother: in registers when one case block holds them all, else in
+            // nvs and ovs
+            float rn[K], ro[K];
+            const bool reg = ncb == 1;
             // level 0 compared once every level-0 item is in (bounded wait)
-            bool l0done = false, fail = false;
+            bool fail = false;
             auto finish_level0 = [&]() {
-                if (l0done) return;
-                l0done = true;
                 if (nev) {
-                    uint32_t spins = 0, got = 0;
-                    while ((got = __shfl_sync(FULL, lane == 0 ? sc[6] : 0u, 0)) < nev && ++spins < d.wait_polls)
+                    uint32_t spins = 0;
+                    bool got = __all_sync(FULL, sc[6] >= nev);
+                    while (!got && ++spins < d.wait_polls) {
                         __nanosleep(64);
-                    if (got < nev) { if (lane == 0) set_status(d.status, ST_TIMEOUT); fail = true; return; }
+                        got = __all_sync(FULL, sc[6] >= nev);
+                    }
+                    if (!got) { if (lane == 0) set_status(d.status, ST_TIMEOUT); fail = true; return; }
                     __threadfence_block();
                 }
                 bool okc = true;
                 for (uint32_t j = lane; j < Cn; j += 32)
                     if (__float_as_uint(nvs[j]) != __float_as_uint(ovs[j])) okc = false;
-                stopped = __all_sync(FULL, okc);
-                stop_level = stopped ? 0 : -1;
-                stopped_w = stopped;
-                stop_level_w = stop_level;
+                stopped_w = __all_sync(FULL, okc);
+                stop_level_w = stopped_w ? 0 : -1;
                 if (root_rec) {
                     float* dst = g.pv_val + (size_t)rslot * Cpad;
                     for (uint32_t j = lane; j < Cpad; j += 32) dst[j] = nvs[j];
@@ -1532,76 +1615,31 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
                     for (uint32_t j = lane; j < Cn; j += 32) dis_case<V>(nvs[j], ovs[j], nd, nf, sq);
                     dis_store<V>(g, i, 0, nd, nf, sq);
                 }
+                if (reg) { load_blk<K>(nvs, 0, rn); load_blk<K>(ovs, 0, ro); }
             };
             if (!anc_ok) { fail = true; if (lane == 0) sc[4] = 1u; }
-            WalkBuilder b;                                 // builder state (lane 0)
-            b.bq = c; b.bqend = c + s; b.bk = 0; b.bpe = (nsmall > 0) ? -1 : A; b.btop = false;
-            const WalkCtx wc{ok_, nsmall, nk, s, r, T, A, hneed, anc, ancg, lvl};
-            bool btop = false;
+            WalkBuilder b;
+            b.bq = c; b.bqend = c + s; b.bk = 0; b.bpe = -1; b.btop = false;
+            const WalkCtx wc{ok_, nsmall, nk, s, r, c, T, me0, tdl, A, hneed, anc, ancg, lvl};
             uint32_t nb = 0, ncm = 0, level = 0;           // levels built, levels combined
             uint32_t rbase = 0, rleft = 0;                 // this child's reserved record slots
-            uint32_t guard = 0;
             if (lane == 0) sc[3] = (uint32_t)A;
-            while (!fail && guard++ < (1u << 24)) {
-                // combine the next level as soon as its sibling values are in;
-                // until then build one more level (the builder's chain of loads
-                // overlaps the evaluators' work instead of delaying the combining)
-                bool ready = false;
-                if (ncm < nb) ready = nev == 0 || __shfl_sync(FULL, lane == 0 ? vcnt[ncm % ring] : 0u, 0) >= ncb;
-                if (!ready) {
-                    uint32_t built = 0;
-                    if (lane == 0 && !b.btop && nb < ncm + ahead) {
-                        LevelDesc& D = desc[nb % ring];
-                        if (build_level(par, wc, b, stopped_w, D)) {
-                            __threadfence_block();
-                            dtag[nb % ring] = nb + 1;
-                            ++nb;
-                            built = 1;
-                            if (D.flags & (LD_BAD | LD_NOSIB)) b.btop = true;
-                        }
-                    }
-                    if (lane == 0) btop = b.btop;
-                    __syncwarp();
-                    nb = __shfl_sync(FULL, nb, 0);
-                    btop = __shfl_sync(FULL, btop ? 1u : 0u, 0) != 0;
-                    if (__shfl_sync(FULL, built, 0)) continue;
-                    if (ncm == nb) {
-                        if (btop) break;                                       // nothing left to combine
-                        continue;
-                    }
+            bool l0done = false;
+            while (!fail) {
+                // keep at least half a ring of levels built ahead of the combination
+                if (!b.btop && nb - ncm <= ring / 2)
+                    nb += build_levels(par, wc, b, stopped_w, desc, dtag, ring, nb, ring - (nb - ncm));
+                // (the first levels are built, and their siblings under way, before level 0 is waited for)
+                if (!l0done) {
+                    l0done = true;
+                    finish_level0();
+                    if (fail) break;
                 }
-                finish_level0();
-                if (fail) break;
+                if (ncm == nb) break;                      // nothing left to combine
                 const uint32_t slot = ncm % ring;
-                LevelDesc D = desc[slot];
-                if (stopped_w && (D.pent >= 0 || D.k > hneed)) break;
-                // the level's sibling values: from the evaluators, or computed here in a team of one
-                if (nev == 0) {
-                    if (!(D.flags & (LD_BAD | LD_NOSIB))) {
-                        for (uint32_t cb = 0; cb < ncb; ++cb) {
-                            float v[K];
-                            if (!stopped_w && D.pent >= 0) {
-                                load_vec<K>(par.slots, Cpad, D.pslot, v, cb);
-                                store_blk<K>(mvs + slot * Cpad, cb, v);
-                            }
-                            if (D.sib >= 0) load_vec<K>(par.slots, Cpad, D.sslot, v, cb);
-                            else {
-                                load_cases<K>(d, cb, ic.xv);
-                                const uint32_t sh = (D.flags & LD_LEFT) ? (uint32_t)tdl : 0u;
-                                eval_run<K, V>(ok_, D.ss - sh, D.se - sh, stA, ic, v, d.status);
-                                if (cb == 0) st_interp += D.se - D.ss;
-                            }
-                            store_blk<K>(svs + slot * Cpad, cb, v);
-                        }
-                    }
-                } else {
-                    uint32_t spins = 0, ready = 0;
-                    while ((ready = __shfl_sync(FULL, lane == 0 ? vcnt[slot] : 0u, 0)) < ncb && ++spins < d.wait_polls)
-                        __nanosleep(64);
-                    if (ready < ncb) { if (lane == 0) set_status(d.status, ST_TIMEOUT); fail = true; break; }
-                    __threadfence_block();
-                }
                 __syncwarp();
+                const LevelDesc D = desc[slot];
+                if (stopped_w && (D.pent >= 0 || D.k > hneed)) break;
                 ++level;
                 if (D.flags & (LD_BAD | LD_NOSIB)) {
                     if (lane == 0) set_error(d, ST_STRUCT, (D.flags & LD_BAD) ? 6 : 7, i, D.p, D.se - D.ss);
@@ -1609,29 +1647,74 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
                     break;
                 }
                 const uint32_t op = D.flags & 0xFFu;
-                const bool left = (D.flags & LD_LEFT) != 0;
-                const float* svl = svs + slot * Cpad;
-                const float* pvv = mvs + slot * Cpad;
+                const bool left = (D.flags & LD_LEFT) != 0, leaf = (D.flags & LD_LEAF) != 0;
+                // the sibling's values: a leaf's at hand, else from the evaluators, or computed here in a team of one
+                if (!leaf) {
+                    if (nev == 0) {
+                        for (uint32_t cb = 0; cb < ncb; ++cb) {
+                            float v[K];
+                            if (D.flags & LD_SLOT) load_vec<K>(par.slots, Cpad, D.sslot, v, cb);
+                            else {
+                                cases(cb);
+                                const uint32_t sh = left ? (uint32_t)tdl : 0u;
+                                eval_run<K, V>(ok_, D.ss - sh, D.se - sh, ic, v, d.status, nullptr);
+                                if (cb == 0) st_interp += D.se - D.ss;
+                            }
+                            store_blk<K>(svs + slot * Cpad, cb, v);
+                        }
+                    } else {
+                        uint32_t spins = 0;
+                        bool ready = __all_sync(FULL, vcnt[slot] >= ncb);
+                        while (!ready && ++spins < d.wait_polls) {
+                            __nanosleep(spins < 64 ? 20 : 64);
+                            ready = __all_sync(FULL, vcnt[slot] >= ncb);
+                        }
+                        if (!ready) { if (lane == 0) set_status(d.status, ST_TIMEOUT); fail = true; break; }
+                        __threadfence_block();
+                    }
+                } else ++st_interp;
                 bool okl = true;
                 uint32_t dnd = 0, dnf = 0;
                 double dsq = 0.0;
-                for (uint32_t j = lane; j < Cpad; j += 32) {
-                    float o[1] = {ovs[j]};
-                    const float sv1[1] = {svl[j]};
-                    combine<1, V>(op, left, o, sv1);         // mother's value at p (exact recomputation)
-                    if (!stopped_w) {
-                        float n1[1] = {nvs[j]};
-                        combine<1, V>(op, left, n1, sv1);
-                        nvs[j] = n1[0];
-                        if (D.pent >= 0) o[0] = pvv[j];
-                        if (j < Cn && __float_as_uint(n1[0]) != __float_as_uint(o[0])) okl = false;
-                        if (g.dis && j < Cn) dis_case<V>(n1[0], o[0], dnd, dnf, dsq);
+                for (uint32_t cb = 0; cb < ncb; ++cb) {
+                    float sv[K];
+                    if (!leaf) load_blk<K>(svs + slot * Cpad, cb, sv);
+                    else {
+                        const uint32_t lop = D.flags >> 24;
+#pragma unroll
+                        for (int k = 0; k < K; ++k) {
+                            const uint32_t j = cb * 32 * K + k * 32 + lane;
+                            if (V == VB) sv[k] = __uint_as_float(mux_word(lop - 4u, mux_pattern(lop - 4u < 5u ? lop - 4u : 0u), j));
+                            else sv[k] = lop == 4 ? d.x[j] : d.consts[lop - 5];
+                        }
                     }
-                    ovs[j] = o[0];
+                    if (!reg) { load_blk<K>(ovs, cb, ro); load_blk<K>(nvs, cb, rn); }
+                    // the mother's value at p (recomputed exactly) and the child's, in one go
+                    float x[2 * K], y[2 * K];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        x[k] = left ? ro[k] : sv[k];
+                        y[k] = left ? sv[k] : ro[k];
+                        x[K + k] = left ? rn[k] : sv[k];
+                        y[K + k] = left ? sv[k] : rn[k];
+                    }
+                    apply_vec<2 * K, V>(op, x, y);
+#pragma unroll
+                    for (int k = 0; k < K; ++k) ro[k] = x[k];
+                    if (!stopped_w) {
+#pragma unroll
+                        for (int k = 0; k < K; ++k) {
+                            rn[k] = x[K + k];
+                            const bool real = cb * 32 * K + k * 32 + lane < Cn;
+                            if (real && __float_as_uint(rn[k]) != __float_as_uint(ro[k])) okl = false;
+                            if (g.dis && real) dis_case<V>(rn[k], ro[k], dnd, dnf, dsq);
+                        }
+                        if (!reg) store_blk<K>(nvs, cb, rn);
+                    }
+                    if (!reg) store_blk<K>(ovs, cb, ro);
                 }
                 const bool lvl_eq = __all_sync(FULL, okl);
                 if (g.dis && !stopped_w) dis_store<V>(g, i, level, dnd, dnf, dsq);
-                __syncwarp();
                 if (!stopped_w) {
                     ++levels_w;
                     ++st_pathops;
@@ -1650,9 +1733,12 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
                     const uint32_t rs = rbase++;
                     --rleft;
                     if (rs >= g.pvcap) { if (lane == 0) set_status(d.status, ST_PATH); fail = true; break; }
-                    const float* src = stopped_w ? ovs : nvs;
                     float* dst = g.pv_val + (size_t)rs * Cpad;
-                    for (uint32_t j = lane; j < Cpad; j += 32) dst[j] = src[j];
+                    if (reg) store_blk<K>(dst, 0, stopped_w ? ro : rn);
+                    else {
+                        const float* src = stopped_w ? ovs : nvs;
+                        for (uint32_t j = lane; j < Cpad; j += 32) dst[j] = src[j];
+                    }
                     if (lane == 0) {
                         g.pv_rec[rs] = make_uint4(i, npv, D.p, rs | (D.pent < 0 ? 0x80000000u : 0u));
                         g.rec_entry[rs] = 0xFFFFFFFFu;
@@ -1662,6 +1748,7 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
                     if (D.pent < 0) ++nins_i;
                 }
                 // release the slot to the builder
+                __syncwarp();
                 if (lane == 0) vcnt[slot] = 0u;
                 __syncwarp();
                 ++ncm;
@@ -1673,56 +1760,54 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
                     g.pv_rec[rbase + k] = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
                     g.rec_entry[rbase + k] = 0xFFFFFFFFu;
                 }
-            // a walk without levels (the child's root is the donated subtree, or
-            // the ancestors failed) still compares level 0
-            if (anc_ok && !fail) finish_level0();
+            if (reg && !fail) store_blk<K>(nvs, 0, rn);
             if (fail && lane == 0) sc[4] = 1u;
             __threadfence_block();
+            __syncwarp();
             if (lane == 0) sc[8] = 1u;                      // evaluators stop
+            if (!fail && !stopped_w) {
+                const float fv = fitness_warp(d, [&](uint32_t j) { return nvs[j]; });
+                if (lane == 0) d.fit[i] = fv;
+            }
         } else {
             // evaluators: each takes the next (level, case block) item in level order from a
-            // shared cursor once the level's descriptor is built, so a long sibling holds up
-            // only the warp evaluating it
+            // shared counter and evaluates it once the level's descriptor is built, so a long
+            // sibling holds up only the warp evaluating it
             for (;;) {
-                uint32_t k = 0, r = 0, fin = 0;
+                uint32_t k = 0, cb = 0, fin = 0;
                 if (lane == 0) {
-                    uint32_t spins = 0;
                     for (;;) {
-                        if (sc[8]) { fin = 1; break; }                  // the combination is over
-                        const unsigned long long c = *reinterpret_cast<volatile unsigned long long*>(cur);
-                        const uint32_t ck = (uint32_t)(c >> 32), cr = (uint32_t)c;
-                        const uint32_t cs = ck % ring;
-                        if (dtag[cs] == ck + 1) {
-                            __threadfence_block();
-                            const unsigned long long nx = (cr + 1 < ncb) ? c + 1 : ((unsigned long long)(ck + 1) << 32);
-                            if (atomicCAS(cur, c, nx) == c) { k = ck; r = cr; break; }
-                            continue;
+                        const uint32_t it = atomicAdd(const_cast<uint32_t*>(&sc[5]), 1u);
+                        k = it / ncb;
+                        cb = it % ncb;
+                        uint32_t spins = 0, tag = 0;
+                        for (;;) {
+                            if (sc[8]) { fin = 1; break; }                  // the combination is over
+                            tag = dtag[k % ring];
+                            if ((tag & 0x7FFFFFFFu) >= k + 1) break;
+                            if (++spins >= d.wait_polls) { set_status(d.status, ST_TIMEOUT); fin = 1; break; }
+                            __nanosleep(spins < 64 ? 20 : 64);
                         }
-                        if (++spins >= d.wait_polls) { set_status(d.status, ST_TIMEOUT); fin = 1; break; }
-                        __nanosleep(64);
+                        // a leaf needs no evaluator (its slot may hold a later level by now)
+                        if (fin || tag == k + 1) break;
                     }
                 }
                 if (__shfl_sync(FULL, fin, 0)) break;
                 k = __shfl_sync(FULL, k, 0);
-                r = __shfl_sync(FULL, r, 0);
-                const uint32_t cb = r;
+                cb = __shfl_sync(FULL, cb, 0);
                 const uint32_t slot = k % ring;
                 __threadfence_block();
-                const LevelDesc D = desc[slot];
-                if (!(D.flags & (LD_BAD | LD_NOSIB))) {
+                const uint32_t ss = desc[slot].ss, se = desc[slot].se, sslot = desc[slot].sslot, fl = desc[slot].flags;
+                if (!(fl & (LD_BAD | LD_NOSIB))) {
                     float v[K];
-                    if (D.pent >= 0) {
-                        load_vec<K>(par.slots, Cpad, D.pslot, v, cb);
-                        store_blk<K>(mvs + slot * Cpad, cb, v);
-                    }
                     bool ab = false;
-                    if (D.sib >= 0) load_vec<K>(par.slots, Cpad, D.sslot, v, cb);
+                    if (fl & LD_SLOT) load_vec<K>(par.slots, Cpad, sslot, v, cb);
                     else {
-                        load_cases<K>(d, cb, ic.xv);
-                        const uint32_t sh = (D.flags & LD_LEFT) ? (uint32_t)tdl : 0u;
+                        cases(cb);
+                        const uint32_t sh = (fl & LD_LEFT) ? (uint32_t)tdl : 0u;
                         // abandoned once the combination is over (the walk stopped below this level)
-                        eval_run<K, V>(ok_, D.ss - sh, D.se - sh, stA, ic, v, d.status, sc + 8, &ab);
-                        if (cb == 0 && !ab) st_interp += D.se - D.ss;
+                        ab = !eval_run<K, V>(ok_, ss - sh, se - sh, ic, v, d.status, sc + 8);
+                        if (cb == 0 && !ab) st_interp += se - ss;
                     }
                     if (ab) break;
                     store_blk<K>(svs + slot * Cpad, cb, v);
@@ -1747,7 +1832,7 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
             __syncthreads();
             continue;
         }
-        // ---- fitness
+        // ---- results
         if (tid == 0) {
             g.stop[i] = stop_level;
             g.plen[i] = levels;
@@ -1758,18 +1843,16 @@ __global__ void __launch_bounds__(MAXT, 512 / MAXT) k_walk(DevPop d, GenBufs g, 
             if (stopped) {
                 d.fit[i] = g.pfit[m];
                 ++st_stopped;
-            } else {
-                d.fit[i] = fitness_of(d, [&](uint32_t j) { return nvs[j]; });
             }
             st_levels += levels;
         }
         __syncthreads();                     // nvs and the shared words are reused by the next child
     }
-    if (lane == 0) atomicAdd(&g.gstat[G_INTERP], st_interp);
+    if (lane == 0) atomicAdd(&g.gstat[G_INTERP], (unsigned long long)st_interp);
     if (tid == 0) {
-        atomicAdd(&g.gstat[G_LEVELS], st_levels);
-        atomicAdd(&g.gstat[G_STOPPED], st_stopped);
-        atomicAdd(&g.gstat[G_PATHOPS], st_pathops);
+        atomicAdd(&g.gstat[G_LEVELS], (unsigned long long)st_levels);
+        atomicAdd(&g.gstat[G_STOPPED], (unsigned long long)st_stopped);
+        atomicAdd(&g.gstat[G_PATHOPS], (unsigned long long)st_pathops);
     }
 }
 
@@ -2155,43 +2238,9 @@ __device__ __forceinline__ uint32_t lower_bound_pos(const uint32_t* e_pos, uint3
     return lo;
 }
 
-// deepest cached ancestor of c in the mother (entry index) or -1
-__device__ __forceinline__ int32_t mother_anchor(const CacheView& par, uint32_t me0, uint32_t me1, uint32_t c,
-                                                 uint32_t r, uint32_t T) {
-    if (c == 0) return -1;
-    int32_t e;
-    if (r >= T) {
-        e = find_exact(par.e_pos, me0, me1, c);
-        return e >= 0 ? par.e_par[e] : -1;
-    }
-    e = find_last_lt(par.e_pos, me0, me1, c);
-    uint32_t guard = 0;
-    while (e >= 0 && par.e_end[e] <= c && guard++ < (1u << 24)) e = par.e_par[e];
-    return e;
-}
-
 __device__ __forceinline__ bool drops(const CacheView& par, int32_t e, int32_t delta, uint32_t T) {
     const uint32_t pos = par.e_pos[e];
     return pos > 0 && (int64_t)par.e_end[e] + delta - (int64_t)pos < (int64_t)T;
-}
-
-// Warp-collective: first index in [lo, hi) of the sorted array a with
-// a[i] >= x (hi if none), by 32-way splitting (two rounds for 1,000 entries).
-__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* a, uint32_t lo, uint32_t hi, uint32_t x) {
-    const uint32_t lane = (uint32_t)lane_id();
-    while (hi - lo > 32) {
-        const uint32_t step = (hi - lo + 31) / 32;
-        const uint32_t last = min(lo + (lane + 1) * step, hi) - 1;     // last index of this lane's segment
-        const uint32_t m = __ballot_sync(FULL, a[last] >= x);
-        if (!m) return hi;
-        const uint32_t f = (uint32_t)__ffs(m) - 1;                      // first segment ending at >= x
-        const uint32_t nlo = lo + f * step;
-        hi = min(nlo + step, hi);
-        lo = nlo;
-    }
-    const uint32_t i = lo + lane;
-    const uint32_t m = __ballot_sync(FULL, i < hi && a[i] >= x);
-    return m ? lo + (uint32_t)__ffs(m) - 1 : hi;
 }
 
 // deepest cached ancestor of c in the mother (entry index) or -1; warp-collective
@@ -2200,10 +2249,7 @@ __device__ __forceinline__ int32_t warp_mother_anchor(const CacheView& par, uint
     if (c == 0) return -1;
     const uint32_t jc = warp_lower_bound(par.e_pos, me0, me1, c);
     if (r >= T) return (jc < me1 && par.e_pos[jc] == c) ? par.e_par[jc] : -1;
-    int32_t e = (jc > me0) ? (int32_t)(jc - 1) : -1;
-    uint32_t guard = 0;
-    while (e >= 0 && par.e_end[e] <= c && guard++ < (1u << 24)) e = par.e_par[e];
-    return e;
+    return (jc > me0) ? warp_anchor(par, me0, (int32_t)(jc - 1), c) : -1;
 }
 
 // Entry count of each child (a warp per child: its four bound searches are
@@ -2375,7 +2421,7 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
         const uint32_t kept = (uint32_t)ckept;
         // inserted ancestors before c (few): kept mother entries and inserts before each
         if (tid < 32) {
-            const int32_t anchor = (delta < 0) ? mother_anchor(par, me0, me1, c, g.rsz[i], T) : -1;
+            const int32_t anchor = (delta < 0 && nins_lt) ? warp_mother_anchor(par, me0, me1, c, g.rsz[i], T) : -1;
             for (uint32_t k = lane; k < nins_lt; k += 32) {
                 const uint32_t px = s_ins[k];
                 uint32_t mlt = lower_bound_pos(par.e_pos, me0, jc, px) - me0;

@@ -280,7 +280,7 @@ int setup_items_kernel(gp_pop* pop) {
     if (smem > (size_t)max_optin)
         return fail(pop, GP_EINVAL, "stack_window %u x cases_per_lane %u needs %zu bytes of shared memory per CTA (%d)",
                     pop->d.W, pop->d.K, smem, max_optin);
-    CK(cudaFuncSetAttribute(k_eval_items<K, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(cudaFuncSetAttribute(k_eval_items<K, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin));
     int nb = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_eval_items<K, V>, GP_WARPS * 32, smem));
     if (nb < 1) nb = 1;
@@ -294,7 +294,8 @@ int setup_items_kernel(gp_pop* pop) {
     if (smem_op > (size_t)max_optin)
         return fail(pop, GP_EINVAL, "stack_window %u x cases_per_lane %u needs %zu bytes of shared memory per CTA (%d)",
                     pop->d.W, pop->d.K, smem_op, max_optin);
-    CK(cudaFuncSetAttribute(k_onepass_eval<K, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_op));
+    CK(cudaFuncSetAttribute(k_onepass_eval<K, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            max_optin - 1024));      // (it has a few bytes of its own)
     int nbo = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbo, k_onepass_eval<K, V>, OP_EVAL_WARPS * 32, smem_op));
     if (nbo < 1) nbo = 1;
@@ -303,6 +304,10 @@ int setup_items_kernel(gp_pop* pop) {
     pop->smem_onepass = smem_op;
     return GP_OK;
 }
+
+// The walk's form (k_walk): the one with all its registers for teams of more
+// than 4 warps and where every child has a team at once (4 of 4 warps per SM).
+bool wide_walk(const gp_pop* pop, uint32_t nw) { return nw > 4 || (uint64_t)pop->d.P * nw <= 16ull * pop->nsm; }
 
 // Team size of the incremental walk (warps per child) and its launch
 // shape.  Auto: a team of 4 -- one building and combining warp and three
@@ -317,30 +322,27 @@ int setup_items_kernel(gp_pop* pop) {
 // shared memory the large ones need, so the longest walks start late).
 template <int K, int V>
 int setup_walk_kernel(gp_pop* pop, uint32_t team) {
+    const uint32_t tab = FxTable<K, V>::bytes(pop->d.ncb);
     const uint32_t ovf = pop->d.ovf_warps;      // the walk shares the interpreter's per-warp overflow stacks
     int max_optin = 0;
     CK(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, pop->dev));
-    {
-        size_t s8 = TeamLayout<K>((int)pop->d.W, pop->d.Cpad, 8).total;
-        if (s8 > (size_t)max_optin) s8 = (size_t)max_optin;
-        CK(cudaFuncSetAttribute(k_walk<K, V, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s8));
-    }
-    const size_t smem16 = TeamLayout<K>((int)pop->d.W, pop->d.Cpad, 16).total;
-    const bool can16 = smem16 <= (size_t)max_optin;
-    if (can16)
-        CK(cudaFuncSetAttribute(k_walk<K, V, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem16));
+    // the attribute belongs to the function, not to the population: the most a CTA may have, so that populations of
+    // different shapes can be created in any order
+    CK(cudaFuncSetAttribute(k_walk<K, V, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin));
+    CK(cudaFuncSetAttribute(k_walk<K, V, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin));
+    const bool can16 = TeamLayout<K>((int)pop->d.W, pop->d.Cpad, 16, tab).total <= (size_t)max_optin;
     auto shape = [&](uint32_t nw, int& grid, size_t& smem) -> int {
-        smem = TeamLayout<K>((int)pop->d.W, pop->d.Cpad, nw).total;
+        smem = TeamLayout<K>((int)pop->d.W, pop->d.Cpad, nw, tab).total;
         int nb = 0;
-        if (nw > 8) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk<K, V, 512>, (int)nw * 32, smem));
-        else CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk<K, V, 256>, (int)nw * 32, smem));
+        if (wide_walk(pop, nw)) CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk<K, V, 512>, (int)nw * 32, smem));
+        else CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk<K, V, 128>, (int)nw * 32, smem));
         if (nb < 1) nb = 1;
         grid = nb * pop->nsm;
         return GP_OK;
     };
     uint32_t nw = team;
     if (!nw) nw = 4;
-    if (TeamLayout<K>((int)pop->d.W, pop->d.Cpad, nw).total > (size_t)max_optin)
+    if (TeamLayout<K>((int)pop->d.W, pop->d.Cpad, nw, tab).total > (size_t)max_optin)
         return fail(pop, GP_EINVAL, "a walk team of %u warps with stack_window %u does not fit shared memory", nw, pop->d.W);
     int grid = 0;
     size_t smem = 0;
@@ -387,7 +389,7 @@ bool wide_fits(const gp_config& cfg) {
     const int W = cfg.stack_window ? (int)cfg.stack_window : 16;
     const uint32_t ncb = (cfg.n_cases + 127) / 128, team = cfg.walk_team ? cfg.walk_team : 4u;
     return ItemsLayout<4, VF>::total(W, ncb) <= (size_t)optin && OnePassEvalLayout<4>::total(W) <= (size_t)optin &&
-           TeamLayout<4>(W, ncb * 128, team).total <= (size_t)optin;
+           TeamLayout<4>(W, ncb * 128, team, FxTable<4, VF>::bytes(ncb)).total <= (size_t)optin;
 }
 
 template <int K, int V>
@@ -1493,13 +1495,12 @@ int launch_walk(gp_pop* pop, const CacheView& par) {
         lc.numAttrs = 1;
         const GenBufs& gb = pop->gb;
         const uint32_t nwl = pop->walk_long_nw;
-        if (nwl > 8) CK(cudaLaunchKernelEx(&lc, k_walk<K, V, 512>, d, gb, par, nwl, wl));
-        else CK(cudaLaunchKernelEx(&lc, k_walk<K, V, 256>, d, gb, par, nwl, wl));
+        CK(cudaLaunchKernelEx(&lc, k_walk<K, V, 512>, d, gb, par, nwl, wl));      // 16 warps, or 8
         CK(cudaEventRecord(pop->wjoin_ev, pop->side2));
     }
     const WalkRange wn{nl, d.P, (uint32_t)Q_WALK, (uint32_t)pop->grid_walk_long * pop->walk_long_nw};
-    k_walk<K, V, 256><<<pop->grid_walk, pop->walk_nw * 32, pop->smem_walk, pop->stream>>>(d, pop->gb, par,
-                                                                                         pop->walk_nw, wn);
+    auto teams = wide_walk(pop, pop->walk_nw) ? k_walk<K, V, 512> : k_walk<K, V, 128>;
+    teams<<<pop->grid_walk, pop->walk_nw * 32, pop->smem_walk, pop->stream>>>(d, pop->gb, par, pop->walk_nw, wn);
     if (nl) CK(cudaStreamWaitEvent(pop->stream, pop->wjoin_ev, 0));
     if (op) CK(cudaStreamWaitEvent(pop->stream, pop->ojoin_ev, 0));
     return GP_OK;
