@@ -559,6 +559,61 @@ __device__ __forceinline__ bool fx_run(LD ld, uint32_t s, uint32_t e, uint32_t w
     return ok && cy.B == 1;
 }
 
+// fx_run over a whole tree [0, e) that also hands out the values of chosen
+// nodes: cap(k) is called by the whole warp when a holds the value of the
+// subtree at pos(k); the positions pos(0) > pos(1) > ... (ncap of them) are
+// functions, or the root.  The instruction list is interrupted after each
+// (its buffer holds FX_CAP_BYTES).
+#define FX_CAP_BYTES ((2 * FX_CHUNK + 2) * 8)
+template <int K, int V, typename LD, typename PosF, typename CapF>
+__device__ __forceinline__ bool fx_run_capture(LD ld, uint32_t e, const FxCtx<K>& c, float (&a)[K], uint32_t ncap, PosF pos,
+                                               CapF cap) {
+    const int lane = lane_id();
+    int32_t base = (int32_t)((e - 1) & ~(uint32_t)(FX_CHUNK - 1));
+    FxCarry cy;
+    cy.w = fx_word(ld, base + 4 * lane, 0u, e);
+    uint32_t wl = fx_word(ld, base - FX_CHUNK + 4 * lane, 0u, e);
+    cy.f = fx_funcs(cy.w);
+    cy.rw = 0xFFFFFFFFu;
+    cy.rf = 0u;
+    cy.B = 0;
+    uint32_t sa = c.stack, lo = 0, k = 0;
+    int32_t nextp = ncap ? (int32_t)pos(0) : -1;
+    bool ok = true;
+    FxHave have;
+#pragma unroll
+    for (int j = 0; j < K; ++j) a[j] = 0.f;
+    for (;;) {
+        const uint32_t fl = fx_funcs(wl);
+        const uint32_t wn = fx_word(ld, base - 2 * FX_CHUNK + 4 * lane, 0u, e);     // in flight during this chunk
+        uint32_t caps = 0, n = 0;
+        while (nextp >= base) {
+            if ((nextp - base) >> 2 == lane) caps |= 1u << (8 * (nextp & 3));
+            ++n;
+            nextp = (k + n < ncap) ? (int32_t)pos(k + n) : -1;
+        }
+        const FxChunk ch = fx_decode<V, true, FxTable<K, V>::row>(cy, fl, base, 0u, e, c.code, c.lt, caps);
+        if (ch.bad) { ok = false; break; }
+        const bool fits = fx_fit<K>(ch, c, lo, sa, ok, have);
+        if (!ok) break;
+        uint32_t ip = c.code;
+        for (uint32_t j = 0;; ++j) {
+            if (fits) fx_exec<K, V>(ip, a, sa, c.x, c.lo);
+            else fx_exec_global<K, V>(ip, a, lo, c);
+            if (j == n) break;
+            cap(k + j);
+        }
+        k += n;
+        __syncwarp();
+        if (base <= 0) break;
+        base -= FX_CHUNK;
+        cy.w = wl;
+        cy.f = fl;
+        wl = wn;
+    }
+    return ok && cy.B == 1;
+}
+
 // this lane's words of the run's last chunk and of the one before it
 template <typename LD>
 __device__ __forceinline__ void fx_first(LD ld, uint32_t s, uint32_t e, uint32_t& w0, uint32_t& w1) {

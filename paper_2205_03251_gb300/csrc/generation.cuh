@@ -1878,10 +1878,9 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, Ge
 // (the deepest stack of the right-to-left scan is max S + 1 <= n / 2 + 1
 // entries: the one-pass warps have overflow stacks that deep of their own,
 // so they run beside the walk).  k_onepass_eval (a warp per child
-// and case block, CTAs of 4 warps) interprets the child a piece of
-// OP_CHUNK bytes at a time and writes each recorded ancestor's values as
-// the scan passes it; the
-// warp that completes a child's last case block writes its fitness.  Which
+// and case block) interprets the child, its words read straight from its
+// parents, and writes each recorded ancestor's values as the scan passes it;
+// the warp that completes a child's last case block writes its fitness.  Which
 // children take this path is decided at crossover (size at most
 // onepass_max, not a clone); the walk skips them.  Disruption recording
 // walks every child.
@@ -1890,20 +1889,17 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, Ge
 #define ONEPASS_DEPTH (ONEPASS_MAX / 2 + 4)   // overflow stack entries per one-pass warp
 #define ONEPASS_WARPS 4                  // warps per CTA of the plan kernel
 #define OP_STAGE (2 * STAGE_BYTES)       // staged bytes per warp of the plan kernel (a whole child)
-#define OP_EVAL_WARPS 4                  // warps per CTA of k_onepass_eval
-#define OP_CHUNK 1024                    // bytes of a child staged at a time by k_onepass_eval
-#define OP_CTAS_PER_SM 6                 // at most this many k_onepass_eval CTAs per SM (24 warps)
+#define OP_EVAL_WARPS 8                  // warps per CTA of k_onepass_eval
+#define OP_CTAS_PER_SM 3                 // at most this many k_onepass_eval CTAs per SM (24 warps)
 
-// Shared memory of a k_onepass_eval CTA: the constant and Boolean-input
-// tables, then per warp a staged piece of the child (OP_CHUNK bytes, at
-// least four stack entries so that a malformed run's underflow stays in the
-// warp's own region) followed by its stack window.  Staging the child a
-// piece at a time (instead of whole) leaves room for more warps per SM.
-template <int K>
+// Shared memory of a k_onepass_eval CTA: the leaf table, then per warp its
+// stack window and the instruction list of a chunk with captures.
+template <int K, int V>
 struct OnePassEvalLayout {
-    static constexpr size_t stage_bytes = (OP_CHUNK > 4 * 32 * K * 4) ? OP_CHUNK : 4 * 32 * K * 4;
-    __host__ __device__ static size_t warp_bytes(int W) { return stage_bytes + SmemLayout<K>::stack_bytes(W); }
-    __host__ __device__ static size_t total(int W) { return SmemLayout<K>::kc_bytes + OP_EVAL_WARPS * warp_bytes(W); }
+    __host__ __device__ static size_t warp_bytes(int W) { return SmemLayout<K>::stack_bytes(W) + FX_CAP_BYTES; }
+    __host__ __device__ static size_t total(int W, uint32_t ncb) {
+        return FxTable<K, V>::bytes(ncb) + OP_EVAL_WARPS * warp_bytes(W);
+    }
 };
 
 struct OnePassSmem {
@@ -1912,28 +1908,28 @@ struct OnePassSmem {
     uint16_t anc[ONEPASS_WARPS][ONEPASS_MAX / 2 + 8];   // ancestors of c (function nodes), nearest first
 };
 
-// Assemble bytes [lo, hi) of child i (lo a multiple of 16, hi - lo <=
-// OP_CHUNK) in `stage` (warp-collective), as stage_child below does for
-// the whole child.
-__device__ __forceinline__ void stage_child_piece(const DevPop& d, const GenBufs& g, uint32_t i, uint32_t nk,
-                                                  uint32_t lo, uint32_t hi, uint8_t* stage) {
-    const int lane = lane_id();
-    __syncwarp();
-    if (g.lazy) {
-        const uint32_t m = g.mother[i];
-        const uint8_t* mb = d.arena + (size_t)g.pbuf[m] * d.cap;
-        const bool clone = (g.flags[i] & F_CLONE) != 0;
-        const uint32_t c = clone ? nk : g.cpos[i], r = clone ? 0 : g.rsz[i], s = clone ? 0 : g.ssz[i];
-        const uint8_t* fr = g.frag + (clone ? 0 : g.frag_off[i]);
-        const uint32_t q0 = lo / 16, q1 = (hi + 15) / 16;
-        for (uint32_t q = q0 + lane; q < q1; q += 32)
-            reinterpret_cast<uint4*>(stage)[q - q0] = child_quad(mb, fr, 16 * q, c, r, s, nk);
-    } else {
-        stage_issue(stage, d.arena + (size_t)d.buf[i] * d.cap, lo, hi);
-        cp_async_commit();
-        cp_async_wait<0>();
+// Four bytes from any address (two aligned loads).
+__device__ __forceinline__ uint32_t load4u(const uint8_t* p) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    const uint32_t* A = reinterpret_cast<const uint32_t*>(a & ~(uintptr_t)3);
+    return __funnelshift_r(__ldg(A), __ldg(A + 1), 8u * (uint32_t)(a & 3u));
+}
+
+// The word at position q (a multiple of 4) of a child that is not built: from
+// its mother's head, the donated fragment fr, or her tail.
+__device__ __forceinline__ uint32_t child_word(const uint8_t* __restrict__ om, const uint8_t* __restrict__ fr, uint32_t q,
+                                               uint32_t c, uint32_t r, uint32_t s, uint32_t nk) {
+    if (q + 4 <= c) return __ldg(reinterpret_cast<const uint32_t*>(om + q));
+    if (q >= c + s) return load4u(om + (q - s + r));
+    if (q >= c && q + 4 <= c + s) return load4u(fr + (q - c));
+    uint32_t w = 0;
+#pragma unroll 1
+    for (uint32_t t = 0; t < 4; ++t) {
+        const uint32_t x = q + t;
+        const uint32_t v = x < c ? om[x] : x < c + s ? fr[x - c] : x < nk ? om[x - s + r] : 0u;
+        w |= v << (8 * t);
     }
-    __syncwarp();
+    return w;
 }
 
 // Assemble child i's bytes [0, nk) in `stage` (warp-collective): from its
@@ -2106,8 +2102,13 @@ __global__ void __launch_bounds__(ONEPASS_WARPS * 32) k_onepass_plan(DevPop d, G
     }
 }
 
+// Bound by the interpreter's indirect branches and, for small children, by
+// the chain of loads before the first word.  4,096 uneven trees x 48 cases
+// 0.58 -> 0.25 ms, 2,048 over the 6-multiplexer 0.51 -> 0.22 ms, 500 ramped
+// trees 67 -> 33 us against the interpreter that took node by node from
+// pieces staged in shared memory.
 template <int K, int V>
-__global__ void __launch_bounds__(OP_EVAL_WARPS * 32, 1) k_onepass_eval(DevPop d, GenBufs g) {
+__global__ void __launch_bounds__(OP_EVAL_WARPS * 32, 3) k_onepass_eval(DevPop d, GenBufs g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // CTAs beyond one warp per unit leave at once (most generations of large
     // trees have few children this small); one thread decides for the CTA
@@ -2119,21 +2120,19 @@ __global__ void __launch_bounds__(OP_EVAL_WARPS * 32, 1) k_onepass_eval(DevPop d
     }
     __syncthreads();
     if ((unsigned long long)blockIdx.x * OP_EVAL_WARPS >= s_units) return;
-    float* kc = reinterpret_cast<float*>(smem_raw);
     const int lane = lane_id(), warp = threadIdx.x >> 5;
-    fill_kc(kc, d.consts);
-    fill_kb(kc + 256);
+    FxTable<K, V>::fill(reinterpret_cast<float*>(smem_raw), d.consts, d.ncb);
     __syncthreads();
-    uint8_t* const stage = smem_raw + SmemLayout<K>::kc_bytes + (size_t)warp * OnePassEvalLayout<K>::warp_bytes((int)d.W);
-    Ictx<K> ic;
-    ic.s = reinterpret_cast<float*>(stage + OnePassEvalLayout<K>::stage_bytes);
-    ic.W = (int)d.W;
-    ic.kc = kc;
-    ic.kb = kc + 256;
-    const uint32_t gwarp = blockIdx.x * OP_EVAL_WARPS + warp;
+    const uint32_t sm = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    const uint32_t wb = sm + FxTable<K, V>::bytes(d.ncb) + warp * (uint32_t)OnePassEvalLayout<K, V>::warp_bytes((int)d.W);
+    FxCtx<K> ic;
+    ic.stack = wb + lane * K * 4;
+    ic.code = wb + (uint32_t)SmemLayout<K>::stack_bytes((int)d.W);
+    ic.lo = lane * K * 4;
+    ic.W = d.W;
     // a child of at most ONEPASS_MAX nodes needs at most ONEPASS_MAX / 2 + 1 stack entries
-    ic.maxd = (int)d.W + ONEPASS_DEPTH;
-    ic.g = g.ovf_op + (size_t)gwarp * ONEPASS_DEPTH * 32 * K;
+    ic.maxd = ONEPASS_DEPTH;
+    ic.g = g.ovf_op + (size_t)(blockIdx.x * OP_EVAL_WARPS + warp) * ONEPASS_DEPTH * 32 * K;
     const uint32_t ncb = d.ncb, Cpad = d.Cpad;
     unsigned long long st_interp = 0;
     // units (child, case block) from the largest size bucket down: the longest
@@ -2155,28 +2154,22 @@ __global__ void __launch_bounds__(OP_EVAL_WARPS * 32, 1) k_onepass_eval(DevPop d
         i = __shfl_sync(FULL, i, 0);
         cb = __shfl_sync(FULL, cb, 0);
         const uint32_t nk = d.size[i];
-        load_cases<K>(d, cb, ic.xv);
-        Istate<K> st;
-#pragma unroll
-        for (int k = 0; k < K; ++k) st.acc[k] = 0.f;
-        st.sp = 0;
-        st.ok = true;
+        load_cases<K>(d, cb, ic.x);
+        ic.lt = FxTable<K, V>::at(sm, cb);
         const uint32_t base = g.op_base[i], R = g.pv_cnt[i];
+        const uint32_t m = g.mother[i], c = g.cpos[i], r = g.rsz[i], s = g.ssz[i];
+        const uint8_t* own = d.arena + (size_t)(g.lazy ? g.pbuf[m] : d.buf[i]) * d.cap;
+        const uint8_t* fr = g.frag + g.frag_off[i];
+        float a[K];
+        auto ld = [&](uint32_t q) {
+            return g.lazy ? child_word(own, fr, q, c, r, s, nk) : __ldg(reinterpret_cast<const uint32_t*>(own + q));
+        };
         auto pos = [&](uint32_t k) { return g.pv_rec[base + k].z; };
-        auto cap = [&](uint32_t k) { store_blk<K>(g.pv_val + (size_t)(base + k) * Cpad, cb, st.acc); };
-        CaptureCursor cur{0u, R ? (int32_t)pos(0) : -1};
-        bool under = false;
-        // the child a piece at a time, right to left (pieces end on multiples of OP_CHUNK)
-        for (uint32_t hi = nk; hi > 0;) {
-            const uint32_t lo = (hi - 1) & ~(uint32_t)(OP_CHUNK - 1);
-            stage_child_piece(d, g, i, nk, lo, hi, stage);
-            interp_capture_range<K, V>(stage, lo, hi, st, ic, R, cur, under, pos, cap);
-            hi = lo;
-        }
-        if (under || st.sp != 1) st.ok = false;
-        if (!st.ok && lane == 0) set_status(d.status, ST_STACK);
+        auto cap = [&](uint32_t k) { store_blk<K>(g.pv_val + (size_t)(base + k) * Cpad, cb, a); };
+        const bool ok = fx_run_capture<K, V>(ld, nk, ic, a, R, pos, cap);
+        if (!ok && lane == 0) set_status(d.status, ST_STACK);
         float* row = g.small_val + (size_t)i * Cpad;
-        store_blk<K>(row, cb, st.acc);
+        store_blk<K>(row, cb, a);
         if (cb == 0) st_interp += nk;
         // the warp that completes the child's last case block writes its fitness
         __threadfence();

@@ -290,7 +290,7 @@ int setup_items_kernel(gp_pop* pop) {
     pop->grid_skel = (nb < 1 ? 1 : nb) * pop->nsm;
     // the one-pass interpreter: CTAs of OP_EVAL_WARPS warps, as many as fit
     // (at most OP_CTAS_PER_SM per SM), each warp with its own overflow stack
-    const size_t smem_op = OnePassEvalLayout<K>::total((int)pop->d.W);
+    const size_t smem_op = OnePassEvalLayout<K, V>::total((int)pop->d.W, pop->d.ncb);
     if (smem_op > (size_t)max_optin)
         return fail(pop, GP_EINVAL, "stack_window %u x cases_per_lane %u needs %zu bytes of shared memory per CTA (%d)",
                     pop->d.W, pop->d.K, smem_op, max_optin);
@@ -388,7 +388,7 @@ bool wide_fits(const gp_config& cfg) {
     }
     const int W = cfg.stack_window ? (int)cfg.stack_window : 16;
     const uint32_t ncb = (cfg.n_cases + 127) / 128, team = cfg.walk_team ? cfg.walk_team : 4u;
-    return ItemsLayout<4, VF>::total(W, ncb) <= (size_t)optin && OnePassEvalLayout<4>::total(W) <= (size_t)optin &&
+    return ItemsLayout<4, VF>::total(W, ncb) <= (size_t)optin && OnePassEvalLayout<4, VF>::total(W, ncb) <= (size_t)optin &&
            TeamLayout<4>(W, ncb * 128, team, FxTable<4, VF>::bytes(ncb)).total <= (size_t)optin;
 }
 
