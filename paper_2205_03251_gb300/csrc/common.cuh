@@ -6,7 +6,6 @@
 #define GP_B 1024            // structure block: positions per warp pass (32 per lane)
 #define GP_NCONST 251        // ephemeral constant table
 #define GP_WARPS 8           // warps per CTA in the persistent kernels
-#define FREE_TILE 4096       // slots per CTA in the free-slot scan
 #define SLOT_NEW 0xFFFFFFFFu // cache entry whose value slot is assigned later in the generation
 #define FULL 0xFFFFFFFFu
 
@@ -66,7 +65,7 @@ struct DevPop {
     float* slots;        // [Scap][Cpad]
     uint32_t* live;      // [Scap] generation stamp of the last cache that referenced the slot
     uint32_t* freeslot;  // [Scap] free slots in slot order (first ones used for new values)
-    uint32_t* ftile;     // [Scap / FREE_TILE + 1] free slots per tile, then their exclusive prefix
+    uint32_t* ftile;     // [1] free slots found for new values
     float* ovf;          // interpreter stack overflow, per warp
     uint32_t* status;    // [1]
     uint32_t* errinfo;   // [4] first failure: site, individual, position, detail

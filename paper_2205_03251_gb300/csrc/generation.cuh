@@ -2,6 +2,8 @@
 // incremental evaluation of the children with failed disruption
 // propagation (Sec. 5, Sec. 6.2, Sec. 6.3, Fig. 1-3).
 #pragma once
+#include <cooperative_groups.h>
+
 #include "fused.cuh"
 #include "structure.cuh"
 #include "mlp.cuh"
@@ -250,15 +252,23 @@ __device__ uint32_t warp_subtree_size_at(const CacheView& par, uint32_t t, const
     return n - x;     // unreachable for well-formed trees
 }
 
+// Warp-collective: the draws of a tournament on the lanes at once (their
+// random loads in one round trip), the earliest draw of the lowest error wins.
 __device__ __forceinline__ uint32_t tournament(const float* fit, uint32_t P, uint32_t T, uint64_t seed,
                                                uint32_t gen, uint32_t child, uint32_t kbase) {
-    uint32_t best = 0;
+    uint32_t best = 0, at = 0xFFFFFFFFu;
     float bf = 0.f;
-    for (uint32_t j = 0; j < T; ++j) {
-        uint32_t idx = (uint32_t)below(draw(seed, gen, child, kbase + j), P);
+    for (uint32_t j = (uint32_t)lane_id(); j < T; j += 32) {
+        const uint32_t idx = (uint32_t)below(draw(seed, gen, child, kbase + j), P);
         float f = fit[idx];
         if (isnan(f)) f = __int_as_float(0x7F800000);
-        if (j == 0 || f < bf) { best = idx; bf = f; }
+        if (at == 0xFFFFFFFFu || f < bf) { best = idx; bf = f; at = j; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const uint32_t ob = __shfl_xor_sync(FULL, best, o), oa = __shfl_xor_sync(FULL, at, o);
+        const float of = __shfl_xor_sync(FULL, bf, o);
+        if (oa != 0xFFFFFFFFu && (at == 0xFFFFFFFFu || of < bf || (of == bf && oa < at))) { best = ob; bf = of; at = oa; }
     }
     return best;
 }
@@ -2305,7 +2315,7 @@ __global__ void __launch_bounds__(1024) k_merge_offsets(DevPop d, GenBufs g) {
 // the child shares, or (bit 31 set) a walk record whose new value gets a
 // free slot of the pool later (k_copy_values).
 __device__ __forceinline__ void put_entry(const DevPop& d, GenBufs& g, uint32_t x, uint32_t pos, uint32_t end,
-                                          uint32_t tree, uint32_t src) {
+                                          uint32_t tree, uint32_t src, uint32_t stamp) {
     d.e_pos[x] = pos;
     d.e_end[x] = end;
     d.e_tree[x] = tree;
@@ -2313,6 +2323,7 @@ __device__ __forceinline__ void put_entry(const DevPop& d, GenBufs& g, uint32_t 
     d.e_c1[x] = -1;
     d.e_par[x] = -1;
     d.e_slot[x] = (src & 0x80000000u) ? SLOT_NEW : src;
+    if (src < d.Scap) d.live[src] = stamp;               // (a new value has bit 31 set)
     if (src & 0x80000000u) g.rec_entry[src & 0x7FFFFFFFu] = x;
 }
 
@@ -2342,7 +2353,7 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
     __shared__ uint64_t cins, ckept;
     const uint32_t tid = threadIdx.x, nthr = blockDim.x;
     const int lane = lane_id();
-    const uint32_t T = d.T;
+    const uint32_t T = d.T, stamp = *g.stamp;
     for (uint32_t i = blockIdx.x; i < d.P; i += gridDim.x) {
         if (g.lazy && !g.sel[i]) continue;                      // uniform per CTA
         const uint32_t o = d.e_off[i];
@@ -2351,7 +2362,7 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
         if (g.flags[i] & F_CLONE) {
             for (uint32_t k = tid; k < me1 - me0; k += nthr) {
                 const uint32_t e = me0 + k;
-                put_entry(d, g, o + k, par.e_pos[e], par.e_end[e], i, par.e_slot[e]);
+                put_entry(d, g, o + k, par.e_pos[e], par.e_end[e], i, par.e_slot[e], stamp);
             }
             continue;
         }
@@ -2408,7 +2419,7 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
                     const int32_t h = find_record(g, i, pos);
                     if (h >= 0) src = g.pv_sorted[h].y | 0x80000000u;
                 }
-                put_entry(d, g, x, pos, anc ? (uint32_t)((int64_t)end + delta) : end, i, src);
+                put_entry(d, g, x, pos, anc ? (uint32_t)((int64_t)end + delta) : end, i, src, stamp);
             }
         }
         const uint32_t kept = (uint32_t)ckept;
@@ -2428,14 +2439,14 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
                 const int32_t h = find_record(g, i, px);
                 if (h >= 0) {
                     const uint4 rec = g.pv_sorted[h];
-                    put_entry(d, g, o + mlt + ilt, rec.x, rec.z, i, (rec.y & 0x7FFFFFFFu) | 0x80000000u);
+                    put_entry(d, g, o + mlt + ilt, rec.x, rec.z, i, (rec.y & 0x7FFFFFFFu) | 0x80000000u, stamp);
                 }
             }
             if (rootins && lane == 0) {
                 const int32_t h = find_record(g, i, c);
                 if (h >= 0) {
                     const uint4 rec = g.pv_sorted[h];
-                    put_entry(d, g, o + kept + nins_lt, rec.x, rec.z, i, (rec.y & 0x7FFFFFFFu) | 0x80000000u);
+                    put_entry(d, g, o + kept + nins_lt, rec.x, rec.z, i, (rec.y & 0x7FFFFFFFu) | 0x80000000u, stamp);
                 }
             }
         }
@@ -2443,108 +2454,84 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
         // part 2: father entries in the donated subtree
         for (uint32_t k = tid; k < jds - jd; k += nthr) {
             const uint32_t e = jd + k;
-            put_entry(d, g, o2 + k, par.e_pos[e] - dd + c, par.e_end[e] - dd + c, i, par.e_slot[e]);
+            put_entry(d, g, o2 + k, par.e_pos[e] - dd + c, par.e_end[e] - dd + c, i, par.e_slot[e], stamp);
         }
         // part 3: mother entries after the removed subtree
         const uint32_t o3 = o2 + (jds - jd);
         for (uint32_t k = tid; k < me1 - jcr; k += nthr) {
             const uint32_t e = jcr + k;
             put_entry(d, g, o3 + k, (uint32_t)((int64_t)par.e_pos[e] + delta), (uint32_t)((int64_t)par.e_end[e] + delta),
-                      i, par.e_slot[e]);
+                      i, par.e_slot[e], stamp);
         }
         __syncthreads();              // shared lists are rewritten for the next child
     }
 }
 
-// ---- slot pool: the children's entries share the parents' value slots;
-// slots that no child entry references are free again, and the walk's new
-// values go to the first free ones (in slot order).
+// ---- slot pool: the children's entries share the parents' value slots
+// (marked with the generation's stamp as the entries are written); slots that
+// no child entry references are free again, and the walk's new values go to
+// the first free ones (in slot order).
 
-// Mark the slots the children's cache references with this generation's stamp.
-__global__ void k_mark_live(DevPop d, GenBufs g) {
-    if (halted(d)) return;
-    const uint32_t ne = d.e_off[d.P];
-    if (ne > d.Ecap) return;
-    const uint32_t stamp = *g.stamp;
-    for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < ne; x += gridDim.x * blockDim.x) {
-        const uint32_t sl = d.e_slot[x];
-        if (sl != SLOT_NEW && sl < d.Scap) d.live[sl] = stamp;
-    }
-}
-
-__device__ __forceinline__ uint32_t block_reduce_add(uint32_t v, uint32_t* ws) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-    __syncthreads();
-    if (lane == 0) ws[w] = v;
-    __syncthreads();
-    uint32_t t = 0;
-    for (uint32_t k = 0; k < (blockDim.x >> 5); ++k) t += ws[k];
-    return t;
-}
-
-// Free slots per tile of FREE_TILE slots (1024 threads, four slots each).
-__global__ void __launch_bounds__(1024) k_free_count(DevPop d, GenBufs g) {
-    if (halted(d)) return;
-    __shared__ uint32_t ws[32];
-    const uint32_t stamp = *g.stamp;
-    const uint32_t nt = (d.Scap + FREE_TILE - 1) / FREE_TILE;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        const uint32_t s0 = t * FREE_TILE + 4 * threadIdx.x;
-        uint32_t c = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) c += (s0 + k < d.Scap && d.live[s0 + k] != stamp) ? 1u : 0u;
-        c = block_reduce_add(c, ws);
-        if (threadIdx.x == 0) d.ftile[t] = c;
-    }
-}
-
-// Exclusive prefix of the per-tile counts (one CTA); too few free slots for
-// the walk's new values is a budget error.
-__global__ void __launch_bounds__(1024) k_free_top(DevPop d, GenBufs g) {
-    if (halted(d)) return;
-    __shared__ uint64_t ws[32];
-    __shared__ uint64_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    const uint32_t nt = (d.Scap + FREE_TILE - 1) / FREE_TILE;
-    for (uint32_t base = 0; base < nt; base += blockDim.x) {
-        const uint32_t t = base + threadIdx.x;
-        const uint64_t v = (t < nt) ? d.ftile[t] : 0;
-        const uint64_t o = block_excl_scan(v, ws, &carry);
-        if (t < nt) d.ftile[t] = (uint32_t)o;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        d.ftile[nt] = (uint32_t)min(carry, (uint64_t)0xFFFFFFFFu);     // free slots in all
-        if (carry < min(g.misc[M_PV], g.pvcap)) set_status(d.status, ST_SLOTS);
-    }
-}
-
-// freeslot[r] = the r-th free slot, for the ranks the new values need.
-__global__ void __launch_bounds__(1024) k_free_emit(DevPop d, GenBufs g) {
-    if (halted(d)) return;
-    __shared__ uint64_t ws[32];
-    __shared__ uint64_t carry;
+// freeslot[r] = the r-th free slot, for the ranks the new values need; their
+// number found in ftile[0].  One cluster of FREE_CTAS CTAs scans from the
+// first slot, FREE_PER slots to a thread (131,072 a step), until it has found
+// them; the CTAs' counts go round through distributed shared memory.  The pool
+// has at least as many free slots as there are records besides the entries'
+// own, usually half of it, so one or two steps do, where counting all tiles
+// of the pool, their prefix and the list took three launches (22 us at 4
+// million slots).
+#define FREE_CTAS 8
+#define FREE_THREADS 512
+#define FREE_PER 32
+__global__ void __cluster_dims__(FREE_CTAS, 1, 1) __launch_bounds__(FREE_THREADS) k_free_find(DevPop d, GenBufs g) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    if (halted(d)) return;                                  // (the same for all CTAs: nothing changes the status beside this kernel)
+    __shared__ uint32_t ws[FREE_THREADS / 32];
+    __shared__ uint32_t tots[2][FREE_CTAS];
+    const uint32_t rank = cluster.block_rank(), lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     const uint32_t stamp = *g.stamp;
     const uint32_t need = min(g.misc[M_PV], g.pvcap);
-    const uint32_t nt = (d.Scap + FREE_TILE - 1) / FREE_TILE;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        const uint32_t base = d.ftile[t];
-        if (base >= need) continue;                       // uniform per CTA
-        if (threadIdx.x == 0) carry = base;
-        __syncthreads();
-        const uint32_t s0 = t * FREE_TILE + 4 * threadIdx.x;
-        uint32_t fr[4], c = 0;
+    uint64_t found = 0;
+    uint32_t par = 0;
+    for (uint64_t base = 0; base < d.Scap && found < need; base += (uint64_t)FREE_CTAS * FREE_THREADS * FREE_PER) {
+        const uint64_t s0 = base + (uint64_t)FREE_PER * (rank * FREE_THREADS + threadIdx.x);
+        uint32_t fr = 0;                                    // bit k: slot s0 + k is free
+        if (s0 + FREE_PER <= d.Scap) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { fr[k] = (s0 + k < d.Scap && d.live[s0 + k] != stamp) ? 1u : 0u; c += fr[k]; }
-        uint32_t r = (uint32_t)block_excl_scan(c, ws, &carry);
+            for (int q = 0; q < FREE_PER / 4; ++q) {
+                const uint4 v = *reinterpret_cast<const uint4*>(d.live + s0 + 4 * q);
+                fr |= ((v.x != stamp ? 1u : 0u) | (v.y != stamp ? 2u : 0u) | (v.z != stamp ? 4u : 0u) |
+                       (v.w != stamp ? 8u : 0u)) << (4 * q);
+            }
+        } else {
+            for (int k = 0; k < FREE_PER; ++k)
+                if (s0 + k < d.Scap && d.live[s0 + k] != stamp) fr |= 1u << k;
+        }
+        // exclusive prefix within the CTA, then over the CTAs
+        const uint32_t own = (uint32_t)__popc(fr);
+        uint32_t incl = own;
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (fr[k]) { if (r < need) d.freeslot[r] = s0 + k; ++r; }
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t v = __shfl_up_sync(FULL, incl, o); if (lane >= (uint32_t)o) incl += v; }
+        if (lane == 31) ws[w] = incl;
         __syncthreads();
+        uint32_t before = 0, total = 0;
+        for (uint32_t q = 0; q < FREE_THREADS / 32; ++q) { const uint32_t v = ws[q]; if (q < w) before += v; total += v; }
+        if (threadIdx.x < FREE_CTAS) *cluster.map_shared_rank(&tots[par][rank], threadIdx.x) = total;
+        cluster.sync();
+        uint64_t r = found + before + incl - own;
+        for (uint32_t q = 0; q < FREE_CTAS; ++q) { const uint32_t v = tots[par][q]; if (q < rank) r += v; found += v; }
+        while (fr && r < need) {
+            d.freeslot[r++] = (uint32_t)s0 + (uint32_t)__ffs(fr) - 1u;
+            fr &= fr - 1;
+        }
+        par ^= 1u;
     }
+    if (rank == 0 && threadIdx.x == 0) {
+        d.ftile[0] = (uint32_t)min(found, (uint64_t)need);
+        if (found < need) set_status(d.status, ST_SLOTS);
+    }
+    cluster.sync();                                         // no CTA leaves while another may write to it
 }
 
 // New values of the children's cache (walk records): each record that
@@ -2557,9 +2544,8 @@ __global__ void k_copy_values(DevPop d, GenBufs g, CacheView par) {
     const int lane = lane_id();
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
-    const uint32_t nt = (d.Scap + FREE_TILE - 1) / FREE_TILE;
     const uint32_t nrec = min(g.misc[M_PV], g.pvcap);
-    const uint32_t avail = min(nrec, d.ftile[nt]);
+    const uint32_t avail = min(nrec, d.ftile[0]);
     for (uint32_t r = gw; r < nrec; r += nw) {
         const uint32_t x = g.rec_entry[r];
         if (x >= ne) continue;                           // not an entry of the children's cache

@@ -78,7 +78,7 @@ struct gp_pop {
     float* pool;                      // value slots shared by both cache sets
     uint32_t* live;                   // [pool_cap] live stamps
     uint32_t* freeslot;               // [pool_cap]
-    uint32_t* ftile;                  // [pool_cap / FREE_TILE + 1]
+    uint32_t* ftile;                  // [1]
     uint64_t pool_cap;
     CacheSet sets[2];
     int cur;                          // set of the current population
@@ -104,7 +104,6 @@ struct gp_pop {
     uint8_t* tree_out;                // [cap] device copy of one tree for gp_get_tree
     uint32_t* tree_meta;              // [4] its size and availability
     uint32_t* io_h;                   // [4] pinned host words: status, tree size and availability
-    uint32_t* rank;                   // [P] work-order ranks
     int prio_high;                    // greatest stream priority of the device (the large teams' launch)
     MlpBufs mlp;
     float mlp_lr;
@@ -459,11 +458,10 @@ int ensure_pool(gp_pop* pop, uint64_t want) {
     const size_t Cpad = pop->d.Cpad;
     float* np = nullptr;
     uint32_t *nl = nullptr, *nf = nullptr, *nt = nullptr;
-    const size_t ntile = want / FREE_TILE + 2;
     if (cudaMalloc(&np, want * Cpad * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&nl, want * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc(&nf, want * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&nt, ntile * sizeof(uint32_t)) != cudaSuccess) {
+        cudaMalloc(&nt, 16) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(np); cudaFree(nl); cudaFree(nf); cudaFree(nt);
         return fail(pop, GP_ENOMEM, "allocation of a value pool of %llu slots failed", (unsigned long long)want);
@@ -823,7 +821,7 @@ int gp_pop_create(const gp_config* cfg_in, const float* x, const float* targets,
         DA2(g.nmother, P); DA2(g.nfather, P); DA2(g.ncpos, P); DA2(g.nrsz, P); DA2(g.ndpos, P); DA2(g.nssz, P);
         DA2(g.nflags, P); DA2(g.sel, P); DA2(g.nfree, 1); DA2(g.pref, P);
         DA2(g.walkA, P); DA2(g.nins, P); DA2(g.mb, P); DA2(g.mcnt, P + 1);
-        DA2(g.order, P); DA2(g.gstat, NGSTAT); DA2(pop->rank, P);
+        DA2(g.order, P); DA2(g.gstat, NGSTAT);
         DA2(g.small_cnt, P); DA2(g.small_val, (size_t)P * d.Cpad); DA2(g.onepass, P); DA2(g.op_base, P);
         DA2(g.op_cnt, 2 * OP_BUCKETS); DA2(g.op_bucket, (size_t)OP_BUCKETS * P);
         cudaMemset(g.onepass, 0, sizeof(uint32_t) * P);
@@ -1527,28 +1525,17 @@ int launch_pack(gp_pop* pop, const CacheView& par) {
     const int mb = (d.P + 7) / 8 < pop->nsm * 2 ? (d.P + 7) / 8 : pop->nsm * 2;   // 8 samples per CTA pass
     k_mlp_infer<<<mb, 256, 0, ms>>>(pop->mlp, d.P, pop->mlp.pred_pack);
     pop->pack_launches = 2;
-    const dim3 rg((d.P + 255) / 256, (d.P + RANK_TILE - 1) / RANK_TILE);
-    // the order of the keys, largest first: one CTA for small populations
-    auto rank_order = [&](const float* key) -> int {
-        if (d.P <= RANK_SMALL) {
-            k_rank_small<<<1, 1024, 0, ms>>>(key, d.P, g.order);
-            pop->pack_launches += 1;
-        } else {
-            CK(cudaMemsetAsync(pop->rank, 0, sizeof(uint32_t) * d.P, ms));
-            k_rank_desc<<<rg, 256, 0, ms>>>(key, d.P, pop->rank);
-            k_rank_scatter<<<pb, 256, 0, ms>>>(pop->rank, d.P, g.order);
-            pop->pack_launches += 2;
-        }
-        return GP_OK;
+    // the order of the keys, largest first
+    auto rank_order = [&](const float* key) {
+        k_rank_order<<<(d.P + RANK_KEYS - 1) / RANK_KEYS, 256, 0, ms>>>(key, d.P, g.order);
+        pop->pack_launches += 1;
     };
     if (pop->cfg.packing == GP_PACK_MLP && d.P <= SORT_MAX) {
-        int r = rank_order(pop->mlp.pred_pack);
-        if (r) return r;
+        rank_order(pop->mlp.pred_pack);
     } else if (pop->cfg.packing == GP_PACK_STATIC && d.P <= SORT_MAX) {
         k_static_key<<<pb, 256, 0, ms>>>(d, g, pop->mlp);
         pop->pack_launches += 1;
-        int r = rank_order(pop->mlp.target);
-        if (r) return r;
+        rank_order(pop->mlp.target);
     } else {
         k_order_identity<<<pb, 256, 0, ms>>>(d, g);
         pop->pack_launches += 1;
@@ -1713,10 +1700,7 @@ int gen_incremental(gp_pop* pop) {
     k_entry_parents<<<gt, 256, 0, pop->side3>>>(d, pop->sb);
     k_child_sizes<<<(d.P + 255) / 256, 256, 0, pop->side3>>>(d, g);
     CK(cudaEventRecord(pop->xjoin_ev[1], pop->side3));
-    k_mark_live<<<gt, 256, 0, pop->stream>>>(d, g);
-    k_free_count<<<pop->nsm * 2, 1024, 0, pop->stream>>>(d, g);
-    k_free_top<<<1, 1024, 0, pop->stream>>>(d, g);
-    k_free_emit<<<pop->nsm * 2, 1024, 0, pop->stream>>>(d, g);
+    k_free_find<<<FREE_CTAS, FREE_THREADS, 0, pop->stream>>>(d, g);
     k_copy_values<<<pop->nsm * 16, 256, 0, pop->stream>>>(d, g, par);
     k_check_slots<<<gt, 256, 0, pop->stream>>>(d);
     CK(cudaStreamWaitEvent(pop->stream, pop->xjoin_ev[1], 0));
@@ -1728,9 +1712,9 @@ int gen_incremental(gp_pop* pop) {
     CK(cudaGetLastError());
     // walk (and the large teams), one-pass plan and evaluation, next plan and
     // copies (fitness-first order, 3), walk records (2), merge counts (2),
-    // MLP training (7), merge, links (3), slot pool (6), statistics
+    // MLP training (7), merge, links (3), slot pool (3), statistics
     pop->launches += 1 + (pop->walk_long_n ? 1u : 0u) + (onepass_on(pop) ? 2u : 0u) + (g.lazy ? 3u : 0u) + 2 + 2 + 7 +
-                     1 + 3 + 6 + 1;
+                     1 + 3 + 3 + 1;
     pop->have_children = false;
     g.evaluated = true;
     pop->last_kind = 1;

@@ -457,11 +457,25 @@ __global__ void k_entry_parents(DevPop d, StructBufs sb) {
         if (lane == 0) tp = t31;
         const bool need = valid && tp == tree;
         int32_t par = -1;
-        // inside the chunk, nearest first (values by shuffle)
-        for (uint32_t dl = 1; dl < 32; ++dl) {
-            const uint32_t ve = __shfl_up_sync(FULL, ee, dl);
-            const uint32_t vt = __shfl_up_sync(FULL, tree, dl);
-            if (need && par < 0 && lane >= dl && vt == tree && ve >= ee) par = (int32_t)(e - dl);
+        // inside the chunk: the nearest earlier entry that ends no earlier, by
+        // halving over maxima of the 1, 2, 4, 8 and 16 entries up to each (the
+        // chunk's own root, if it is there, ends last of its tree, so the
+        // search never goes past it into another tree)
+        {
+            uint32_t mx[5];
+            mx[0] = ee;
+#pragma unroll
+            for (int k = 1; k < 5; ++k) {
+                const uint32_t v = __shfl_up_sync(FULL, mx[k - 1], 1 << (k - 1));
+                mx[k] = lane >= (1u << (k - 1)) ? max(mx[k - 1], v) : mx[k - 1];
+            }
+            int at = (int)lane - 1;
+#pragma unroll
+            for (int k = 4; k >= 0; --k) {
+                const uint32_t v = __shfl_sync(FULL, mx[k], at < 0 ? 0 : at);
+                if (at >= 0 && v < ee) at -= 1 << k;          // none among the 2^k entries up to `at`
+            }
+            if (need && at >= 0) par = (int32_t)(ch * 32 + (uint32_t)at);
         }
         // the previous chunk, a ballot per unresolved lane
         uint32_t pend = __ballot_sync(FULL, need && par < 0);
