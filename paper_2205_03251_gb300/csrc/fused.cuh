@@ -9,6 +9,7 @@
 //   f L L    push acc; acc = f(L, L)
 //   f L .    acc = f(L, acc)       the left operand is a leaf, the right one was just evaluated
 //   f f ..   acc = f(acc, pop)     the left operand was just evaluated
+//   f g L L  acc = f(g(L, L), acc) Boolean sets: the left operand has two leaves; neither a push nor a pop
 //   L        push acc; acc = L     a leaf that no function to its left takes at once
 // A node's form depends on its own opcode and its two neighbours' on either
 // side, so 32 lanes decode 128 nodes with a few byte-parallel operations
@@ -40,7 +41,17 @@
 //   16..23 f L .: 16 + 2 f + (left is a constant)
 //   24..27 f f ..: 24 + f
 //   28, 29 L: 28 + (it is a constant)
+//   32..95 f g L L (Boolean): 32 + 16 f + 4 g + 3
 // Boolean: the constant bits are all set.
+//
+// f g L L saves the Boolean sets, whose leaves are all of one kind, a dispatch
+// and a round trip through the stack for 16 more pieces of code (full
+// evaluation of 29.6 M nodes of the 11-multiplexer set 1.71 -> 1.58 ms).  The
+// other sets would need 48 more, whose instruction fetches cost more than the
+// dispatches they save: 0.5 GB of binary32 trees 9.0 -> 14.5 ms, 29 M nodes
+// of integer trees 1.77 -> 1.97 ms.  (And a paired product followed by a paired sum
+// in one piece of code is joined into one rounding by the assembler, also
+// with .rn on both: 22 % of random triples differ.)
 
 __device__ __forceinline__ uint32_t fx_signs(uint32_t v) {      // each byte all ones or zeros by its top bit
     uint32_t r;
@@ -117,8 +128,15 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     const uint32_t n1 = __funnelshift_r(w, wr, 8), n2 = __funnelshift_r(w, wr, 16);      // the next two opcodes
     const uint32_t f1 = __funnelshift_r(f, fr, 8), f2 = __funnelshift_r(f, fr, 16);      // are they functions
     const uint32_t p1 = __funnelshift_l(fl, f, 8), p2 = __funnelshift_l(fl, f, 16);      // the two before
-    // a function always makes an instruction, a leaf when neither node before it takes it
-    const uint32_t head = valid & (f | ~(p1 | p2));
+    // f L L; and f g L L, where g's instruction becomes part of f's (not while values are captured: g may be asked for)
+    const uint32_t isll = f & ~f1 & ~f2;
+    uint32_t pair = 0u, taken = 0u;
+    if (V == VB && !CAP) {
+        pair = f & f1 & ~f2 & ~__funnelshift_r(f, fr, 24);
+        taken = isll & p1;
+    }
+    // a function makes an instruction, a leaf when neither node before it takes it
+    const uint32_t head = valid & ((f & ~taken) | ~(f | p1 | p2));
     // depths: +1 per leaf, -1 per function, summed from the right
     const uint32_t step = (valid & 0x01010101u) | (valid & f);
     const int d3 = __dp4a((int)step, 0x01000000, 0), d2 = __dp4a((int)step, 0x01010000, 0);
@@ -147,13 +165,15 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     r.bad = __any_sync(FULL, r.mn < 0 || tail);
     // instruction indexes of the four bytes at once
     uint32_t idx, A;                     // index; the byte of the first operand
-    uint32_t both = 0;                   // f L L with two table operands
+    uint32_t both, second = n2;          // f L L and f g L L with two table operands; the byte of the second
     if (V == VB) {
         const uint32_t ll = ((w << 2) & 0x0C0C0C0Cu) | 0x03030303u, lf = ((w << 1) & 0x06060606u) | 0x11111111u;
         const uint32_t fp = (w & 0x03030303u) | 0x18181818u;
-        idx = (f & ~f1 & ~f2 & ll) | (f & ~f1 & f2 & lf) | (f & f1 & fp) | (~f & 0x1D1D1D1Du);
-        A = (f & n1) | (~f & w);
-        both = f & ~f1 & ~f2;
+        const uint32_t fg = (((w & 0x03030303u) << 4) + 0x23232323u) | ((n1 << 2) & 0x0C0C0C0Cu);
+        idx = (isll & ll) | (f & ~f1 & f2 & lf) | (f & f1 & ~pair & fp) | (~f & 0x1D1D1D1Du) | (pair & fg);
+        A = (pair & n2) | (f & ~pair & n1) | (~f & w);
+        both = isll | pair;
+        second = (pair & __funnelshift_r(w, wr, 24)) | (~pair & n2);
     } else {
         const uint32_t x = fx_zero_bytes(w ^ 0x04040404u);
         const uint32_t xr = fx_zero_bytes(wr ^ 0x04040404u);
@@ -163,7 +183,6 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
         const uint32_t lf = ((w << 1) & 0x06060606u) | 0x10101010u | (~x1 & 0x01010101u);
         const uint32_t fp = (w & 0x03030303u) | 0x18181818u;
         const uint32_t lp = 0x1C1C1C1Cu | (~x & 0x01010101u);
-        const uint32_t isll = f & ~f1 & ~f2;
         idx = (isll & ll) | (f & ~f1 & f2 & lf) | (f & f1 & fp) | (~f & lp);
         A = (~f & w) | (f & ((isll & x1 & n2) | (~(isll & x1) & n1)));   // the constant: the right leaf when the left one is x
         both = isll & ~x1 & ~x2;
@@ -174,8 +193,8 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
 #pragma unroll
     for (int j = 3; j >= 0; --j) {
         const uint32_t on = head & (1u << (8 * j));
-        const uint32_t second = (lt << 16) + ((n2 >> (8 * j)) & most) * (size << 16);
-        const uint32_t y = lt + ((A >> (8 * j)) & most) * size + ((both & (1u << (8 * j))) ? second : 0u);
+        const uint32_t y2 = (lt << 16) + ((second >> (8 * j)) & most) * (size << 16);
+        const uint32_t y = lt + ((A >> (8 * j)) & most) * size + ((both & (1u << (8 * j))) ? y2 : 0u);
         fx_put(on, at, (idx >> (8 * j)) & 0xFFu, y);
         at += on ? 8u : 0u;
         if (CAP) {
@@ -317,8 +336,17 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     FXLD_##F("n", "t") FXLD_##F("r", "u") FX_NEXT FX_PUSH(F) FXO_##F(ins, "a", "n", "r") post FX_GO                  \
     "FXM" o "1:\n\tadd.u32 t, oy, lo;\n\t" FXLD_##F("n", "t") FX_NEXT FXO_##F(ins, "a", "n", "a") post FX_GO         \
     "FXP" o "0:\n\t" FX_NEXT FX_POP(F) FXO_##F(ins, "a", "a", "r") post FX_GO
+// f g L L
+#define FX_BPAIR(F, fo, go, fi, fpost, gi, gpost)                                                                   \
+    "FXC" fo go ":\n\tand.b32 t, oy, 0xFFFF;\n\tshr.u32 u, oy, 16;\n\tadd.u32 t, t, lo;\n\tadd.u32 u, u, lo;\n\t"     \
+    FXLD_##F("n", "t") FXLD_##F("r", "u") FX_NEXT FXO_##F(gi, "r", "n", "r") gpost FXO_##F(fi, "a", "r", "a") fpost FX_GO
+#define FX_BPAIRS(F, fo, fi, fpost)                                                                                 \
+    FX_BPAIR(F, fo, "0", fi, fpost, "and.b32", "") FX_BPAIR(F, fo, "1", fi, fpost, "or.b32", "")                      \
+    FX_BPAIR(F, fo, "2", fi, fpost, "and.b32", FXNR_##F) FX_BPAIR(F, fo, "3", fi, fpost, "or.b32", FXNR_##F)
 #define FXN_S1 "not.b32 a0, a0;\n\t"
 #define FXN_S2 FXN_S1 "not.b32 a1, a1;\n\t"
+#define FXNR_S1 "not.b32 r0, r0;\n\t"
+#define FXNR_S2 FXNR_S1 "not.b32 r1, r1;\n\t"
 
 #define FX_REGS_S ".reg .b32 a0, a1, x0, x1, r0, r1, n0, n1, c0, c1;\n\t"
 #define FX_REGS_P ".reg .b64 a0, a1, x0, x1, r0, r1, n0, n1, c0, c1, y, z, v, q, one;\n\tmov.b64 one, 0x3F8000003F800000;\n\t"
@@ -329,10 +357,12 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     "FXT: .branchtargets FXA00, FXA01, FXA02, FXA03, FXA10, FXA11, FXA12, FXA13, FXA20, FXA21, FXA22, FXA23, "       \
     "FXA30, FXA31, FXA32, FXA33, FXM00, FXM01, FXM10, FXM11, FXM20, FXM21, FXM30, FXM31, FXP00, FXP10, FXP20, "      \
     "FXP30, FXL0, FXL1, FXEND;\n\t"
+#define FX_BROW4(l) l ", " l ", " l ", " l
+#define FX_BROW(f) FX_BROW4("FXC" f "0") ", " FX_BROW4("FXC" f "1") ", " FX_BROW4("FXC" f "2") ", " FX_BROW4("FXC" f "3")
 #define FX_BTABLE                                                                                                   \
     "FXT: .branchtargets FXA03, FXA03, FXA03, FXA03, FXA13, FXA13, FXA13, FXA13, FXA23, FXA23, FXA23, FXA23, "       \
     "FXA33, FXA33, FXA33, FXA33, FXM01, FXM01, FXM11, FXM11, FXM21, FXM21, FXM31, FXM31, FXP00, FXP10, FXP20, "      \
-    "FXP30, FXL1, FXL1, FXEND;\n\t"
+    "FXP30, FXL1, FXL1, FXEND, FXEND, " FX_BROW("0") ", " FX_BROW("1") ", " FX_BROW("2") ", " FX_BROW("3") ";\n\t"
 #define FX_START "ld.shared.v2.b32 {ix, oy}, [ip];\n\tadd.u32 ip, ip, 8;\n\t" FX_NEXT FX_GO
 #define FX_STOP "FXEND:\n\tsub.u32 ip, ip, 8;\n\t"
 #define FX_LEAVES(F)                                                                                                \
@@ -347,6 +377,8 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
 #define FX_BODY_B(F)                                                                                                \
     FX_BFUNC(F, "0", "and.b32", "") FX_BFUNC(F, "1", "or.b32", "") FX_BFUNC(F, "2", "and.b32", FXN_##F)              \
     FX_BFUNC(F, "3", "or.b32", FXN_##F)                                                                              \
+    FX_BPAIRS(F, "0", "and.b32", "") FX_BPAIRS(F, "1", "or.b32", "") FX_BPAIRS(F, "2", "and.b32", FXN_##F)           \
+    FX_BPAIRS(F, "3", "or.b32", FXN_##F)                                                                             \
     "FXL1:\n\tadd.u32 t, oy, lo;\n\t" FX_NEXT FX_PUSH(F) FXLD_##F("a", "t") FX_GO FX_STOP
 
 // Run the list at shared address `ip` up to an end mark; afterwards ip is
@@ -461,9 +493,16 @@ __device__ __forceinline__ void fx_exec_global(uint32_t& ip, float (&a)[K], uint
     };
     for (;; ip += 8) {
         const uint32_t idx = lds_u32(ip), y = lds_u32(ip + 12);
-        if (idx >= FX_EXIT) break;
+        if (idx == FX_EXIT) break;
         float l[K], r[K];
-        if (idx < 16u) {
+        if (V == VB && idx >= 32u) {
+            leaf(y & 0xFFFFu, true, l);
+            leaf(y >> 16, true, r);
+            apply_vec<K, V>((idx >> 2) & 3u, l, r);
+            apply_vec<K, V>((idx - 32u) >> 4, l, a);
+#pragma unroll
+            for (int k = 0; k < K; ++k) a[k] = l[k];
+        } else if (idx < 16u) {
             const bool ca = idx & 2u, cb = idx & 1u;
             push();
             leaf(ca && cb ? y & 0xFFFFu : y, ca, l);
