@@ -519,7 +519,8 @@ int run_structure(gp_pop* pop) {
     DevPop& d = pop->d;
     const int gthreads = pop->grid_threads;
     k_blk_offsets<<<1, 1024, 0, pop->stream>>>(d);
-    k_unit_flags<<<pop->nsm * 16, FLAG_WARPS * 32, 0, pop->stream>>>(d, pop->sb);
+    if (d.T >= 64) k_unit_flags_wide<<<pop->nsm * 16, FLAG_WARPS * 32, 0, pop->stream>>>(d, pop->sb);
+    else k_unit_flags<<<pop->nsm * 16, FLAG_WARPS * 32, 0, pop->stream>>>(d, pop->sb);
     const int scan_grid = pop->nsm * 2;
     k_scan_tiles<<<scan_grid, SCAN_TILE, 0, pop->stream>>>(d, pop->sb);
     k_scan_top<<<1, SCAN_TILE, 0, pop->stream>>>(d, pop->sb);

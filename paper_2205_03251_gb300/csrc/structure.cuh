@@ -9,7 +9,7 @@
 // rises above b[i] on (i, i+T).  Positions past the end count as leaves.
 //
 // All steps are data parallel:
-//   k_unit_flags    one warp per 1024-position block: flags, per-32-chunk
+//   k_unit_flags    (k_unit_flags_wide for T >= 64) one warp per 1024-position block: flags, per-32-chunk
 //                   balances and maxima (window maxima of width T-1 from
 //                   segmented prefix/suffix maxima over T-aligned segments)
 //   k_scan_*        prefix sums of flag counts and block balances
@@ -188,6 +188,116 @@ __global__ void __launch_bounds__(FLAG_WARPS * 32) k_unit_flags(DevPop d, Struct
             bm = max(bm, __shfl_down_sync(FULL, bm, o));
         }
         if (lane == 0) { sb.u_cnt[u] = cnt; sb.u_total[u] = tot0; sb.u_max[u] = bm; }
+    }
+}
+
+// The same flags for thresholds of at least two 32-position chunks.  A node
+// can head a large subtree only when the largest before-balance of its chunk
+// reaches W, the largest of the T/32 - 1 chunks after it, which few chunks
+// do; the warp then tests the 32 positions of such a chunk at once, each
+// against the rest of the chunk, W, and the start of the chunk that ends the
+// window.  A warp takes up to FLAG_SPAN blocks in a row and computes each block's
+// chunk sums and maxima once (they serve as the next block's too).  Bound by
+// integer instructions; structure pass over 0.5 GB of opcodes: 1.98 ms with the
+// window maxima of every position through shared memory, 1.14 ms.
+#define FLAG_SPAN 8
+__global__ void __launch_bounds__(FLAG_WARPS * 32) k_unit_flags_wide(DevPop d, StructBufs sb) {
+    const int lane = lane_id();
+    const uint32_t nunits = d.blk_off[d.P];
+    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
+    const int L = (int)d.T / 32;                  // chunks per window, 2..32
+    const uint32_t below = (1u << lane) - 1u;
+    // sum, largest before-balance and largest after-balance of a chunk, from its start
+    auto stats = [](uint32_t bits, int& t, int& mb, int& ma) {
+        int a = 0;
+        mb = 0;
+        ma = -64;
+#pragma unroll
+        for (int s = 0; s < 32; ++s) {
+            a += 2 * (int)((bits >> s) & 1u) - 1;
+            ma = max(ma, a);
+            if (s == 30) mb = max(0, ma);
+        }
+        t = a;
+    };
+    const uint32_t span = min((uint32_t)FLAG_SPAN, max(1u, nunits / nw));      // fewer when there are not enough for all warps
+    for (uint32_t us = gw * span; us < nunits; us += nw * span) {
+        const uint32_t ue = min(us + span, nunits);
+        uint32_t tree = find_segment(d.blk_off, d.P, us), next = us;      // next: first block of the following tree
+        uint32_t first = 0, n = 0, b0 = 0;
+        const uint8_t* ops = nullptr;
+        int t0 = 0, mb0 = 0, ma0 = 0;
+        bool have = false;
+        for (uint32_t u = us; u < ue; ++u) {
+            if (!have || u >= next) {
+                while (have && u >= d.blk_off[tree + 1]) ++tree;
+                have = true;
+                first = d.blk_off[tree];
+                next = d.blk_off[tree + 1];
+                ops = tree_ptr(d, tree);
+                n = d.size[tree];
+                b0 = leaf_bits(ops, n, (u - first) * GP_B + 32 * lane);
+                stats(b0, t0, mb0, ma0);
+            }
+            const uint32_t base = (u - first) * GP_B;
+            const uint32_t b1 = leaf_bits(ops, n, base + GP_B + 32 * lane);
+            int t1, mb1, ma1;
+            stats(b1, t1, mb1, ma1);
+            const int i0 = warp_incl_sum(t0), i1 = warp_incl_sum(t1);
+            const int tot0 = __shfl_sync(FULL, i0, 31);
+            const int v0 = i0 - t0, w0 = tot0 + i1 - t1;      // balance before the lane's chunk, this block and the next
+            // x0, x1: largest before-balance of the `width` chunks from the lane's on (both blocks)
+            int x0 = v0 + mb0, x1 = w0 + mb1;
+            const int m0 = x0;
+            auto at = [&](int o) {                            // x of the chunk o after this lane's
+                const int p = __shfl_sync(FULL, x0, (lane + o) & 31), q = __shfl_sync(FULL, x1, (lane + o) & 31);
+                return lane + o < 32 ? p : q;
+            };
+            for (int width = 1; width < L / 2; width *= 2) {
+                const int p = at(width);
+                const int q = __shfl_sync(FULL, x1, (lane + width) & 31);
+                x0 = max(x0, p);
+                if (lane + width < 32) x1 = max(x1, q);
+            }
+            const int pa = at(1), pb = at(L / 2);
+            const int W = max(pa, pb);                        // the L - 1 chunks after the lane's
+            uint32_t pass = __ballot_sync(FULL, m0 >= W && base + 32 * lane < n);
+            uint32_t flags = 0;
+            while (pass) {
+                const int l = __ffs(pass) - 1;
+                pass &= pass - 1;
+                const uint32_t bits = __shfl_sync(FULL, b0, l);
+                const int vv = __shfl_sync(FULL, v0, l), ww = __shfl_sync(FULL, W, l);
+                const int e = l + L;                          // the chunk the windows end in
+                const uint32_t eb0 = __shfl_sync(FULL, b0, e & 31), eb1 = __shfl_sync(FULL, b1, e & 31);
+                const int ev0 = __shfl_sync(FULL, v0, e & 31), ev1 = __shfl_sync(FULL, w0, e & 31);
+                const uint32_t eb = e < 32 ? eb0 : eb1;
+                const int ev = e < 32 ? ev0 : ev1;
+                const int v = vv + 2 * __popc(bits & below) - lane;           // before-balance at position `lane`
+                int y = v, z = ev + 2 * __popc(eb & below) - lane;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int p = __shfl_down_sync(FULL, y, o), q = __shfl_up_sync(FULL, z, o);
+                    if (lane + o < 32) y = max(y, p);
+                    if (lane >= o) z = max(z, q);
+                }
+                int rest = __shfl_down_sync(FULL, y, 1), start = __shfl_up_sync(FULL, z, 1);
+                if (lane == 31) rest = NEG_INF_I;
+                if (lane == 0) start = NEG_INF_I;
+                const uint32_t f = __ballot_sync(FULL, v >= ww && v >= rest && v >= start && base + 32 * l + lane < n);
+                if (lane == l) flags = f;
+            }
+            if (base == 0 && lane == 0 && n > 0) flags |= 1u;   // every root is cached
+            const int cmax = v0 + ma0;
+            sb.u_flags[(size_t)u * 32 + lane] = flags;
+            sb.u_cv0[(size_t)u * 32 + lane] = v0;
+            sb.u_cmax[(size_t)u * 32 + lane] = cmax;
+            const uint32_t cnt = __reduce_add_sync(FULL, (uint32_t)__popc(flags));
+            const int bm = __reduce_max_sync(FULL, cmax);
+            if (lane == 0) { sb.u_cnt[u] = cnt; sb.u_total[u] = tot0; sb.u_max[u] = bm; }
+            b0 = b1; t0 = t1; mb0 = mb1; ma0 = ma1;
+        }
     }
 }
 
