@@ -84,7 +84,9 @@ typedef struct {
     uint32_t cache_threshold;   /* subtree size from which node values are cached, 2..1024 (default 1024) */
     uint32_t tournament;        /* tournament size (default 7) */
     uint32_t packing;           /* GP_PACK_* order of incremental work */
-    uint32_t cases_per_lane;    /* 0 = auto; else 1, 2 or 4 test cases per GPU lane (words for the
+    uint32_t cases_per_lane;    /* 0 = auto (1 up to 32 cases, 4 where more than 64 binary32 cases fill an
+                                   even number of 64-case blocks and shared memory has room, else 2);
+                                   else 1, 2 or 4 test cases per GPU lane (words for the
                                    Boolean sets; 4 only for GP_FP32_ARITH; GP_BOOL_MUX6 uses 1) */
     uint64_t cache_budget_bytes;/* device bytes for cached value vectors (0 = 40 GiB) */
     uint64_t seed;              /* master seed of every stochastic choice */
@@ -423,9 +425,9 @@ int gp_set_profiling(gp_pop* pop, int on);
  *   d_x, d_t   n_cases inputs and targets (1 <= n_cases <= 4096); d_consts 251 floats
  *   d_values   out: n_trees x n_cases root values (row per tree)
  *   d_fitness  out: n_trees fitness values (sum of |value - target| in case order)
- * Same arithmetic as gp_eval_full.  Scratch (the interpreter's deep-stack
- * overflow for 64 warps, a work counter, a status word) lives in one
- * file-scope device array of about 8.5 MB that every GPU loading the library
+ * Same arithmetic as gp_eval_full.  Runs on the whole GPU.  Scratch (64 overflow
+ * stacks, which warps whose stack outgrows the shared window take in turn; a
+ * work counter, a status word) lives in one file-scope device array of about 8.5 MB that every GPU loading the library
  * holds until exit.  The first call on a device (and the first after that
  * device's context was re-created) looks up the array's device address
  * (cudaGetSymbolAddress) with the device current; make that first call
@@ -435,7 +437,8 @@ int gp_set_profiling(gp_pop* pop, int on);
  * synchronises its stream before returning.  Returns GP_EINVAL for bad
  * arguments or a malformed tree, GP_ECAPACITY when a tree is empty, larger
  * than 1023 nodes or outside ops_bytes; *status_out (host, may be NULL) gets
- * the raw flags (1: size or bounds, 2: malformed tree).
+ * the raw flags (1: size or bounds, 2: malformed tree, 4: no overflow
+ * stack came free within the wait limit, returned as GP_ETIMEOUT).
  */
 int gp_eval_small_noalloc(const uint8_t* d_ops, size_t ops_bytes, const uint64_t* d_off, uint32_t n_trees,
                           const float* d_x, const float* d_t, const float* d_consts, uint32_t n_cases,
