@@ -9,7 +9,7 @@
 // rises above b[i] on (i, i+T).  Positions past the end count as leaves.
 //
 // All steps are data parallel:
-//   k_unit_flags    (k_unit_flags_wide for T >= 64) one warp per 1024-position block: flags, per-32-chunk
+//   k_unit_flags    (k_unit_flags_wide for T >= 128) one warp per 1024-position block: flags, per-32-chunk
 //                   balances and maxima (window maxima of width T-1 from
 //                   segmented prefix/suffix maxima over T-aligned segments)
 //   k_scan_*        prefix sums of flag counts and block balances
@@ -191,7 +191,8 @@ __global__ void __launch_bounds__(FLAG_WARPS * 32) k_unit_flags(DevPop d, Struct
     }
 }
 
-// The same flags for thresholds of at least two 32-position chunks.  A node
+// The same flags for thresholds of at least two 32-position chunks (used
+// from four on).  A node
 // can head a large subtree only when the largest before-balance of its chunk
 // reaches W, the largest of the T/32 - 1 chunks after it, which few chunks
 // do; the warp then tests the 32 positions of such a chunk at once, each
