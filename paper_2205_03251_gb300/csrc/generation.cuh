@@ -2494,6 +2494,7 @@ __global__ void __cluster_dims__(FREE_CTAS, 1, 1) __launch_bounds__(FREE_THREADS
     const uint32_t need = min(g.misc[M_PV], g.pvcap);
     uint64_t found = 0;
     uint32_t par = 0;
+    cluster.sync();                                         // every CTA has started before another writes to it
     for (uint64_t base = 0; base < d.Scap && found < need; base += (uint64_t)FREE_CTAS * FREE_THREADS * FREE_PER) {
         const uint64_t s0 = base + (uint64_t)FREE_PER * (rank * FREE_THREADS + threadIdx.x);
         uint32_t fr = 0;                                    // bit k: slot s0 + k is free
