@@ -112,6 +112,7 @@ struct gp_pop {
     uint32_t* gwords;                 // device: [0] = 0, [1] = generations replayed by the captured graph
     cudaGraphExec_t gexec;            // captured generation loop (graph mode)
     uint32_t graph_n;                 // generations per replay
+    int graph_cur;                    // cur when the graph was captured: which buffers it takes for the parents'
     uint32_t graph_launches;          // kernel launches per replay
     cudaStream_t cap_stream;          // private capture stream when the population runs on the legacy stream
     cudaStream_t side;                // second stream: work order (at crossover), copies (beside the cache update)
@@ -656,6 +657,7 @@ int gp_pop_create(const gp_config* cfg_in, const float* x, const float* targets,
     memset(pop->ev_count, 0, sizeof pop->ev_count);
     pop->gexec = nullptr;
     pop->graph_n = 0;
+    pop->graph_cur = 0;
     pop->cap_stream = nullptr;
     pop->side = nullptr;
     pop->side2 = nullptr;
@@ -1115,6 +1117,7 @@ int gp_graph_capture(gp_pop* pop, uint32_t first_generation, uint32_t n_generati
     ce = cudaGraphUpload(pop->gexec, own ? own : 0);
     if (ce != cudaSuccess) { cudaGetLastError(); return fail(pop, GP_ECUDA, "graph upload failed: %s", cudaGetErrorString(ce)); }
     pop->graph_n = n_generations;
+    pop->graph_cur = cur0;
     pop->graph_launches = launches + 1;
     return GP_OK;
 }
@@ -1124,6 +1127,11 @@ int gp_graph_launch(gp_pop* pop) {
     if (!pop->gexec) return fail(pop, GP_ESTATE, "no captured graph (gp_graph_capture)");
     if (!pop->gb.evaluated || pop->have_children)
         return fail(pop, GP_ESTATE, "gp_graph_launch needs an evaluated population with no pending children");
+    // the graph's kernels hold the addresses of the capture: after an odd number of generations the parents are in the
+    // other buffers, whose free list no longer matches
+    if (pop->cur != pop->graph_cur)
+        return fail(pop, GP_ESTATE, "an odd number of generations since the capture: parents and children have changed buffers "
+                                    "(capture again)");
     CK(cudaGraphLaunch(pop->gexec, pop->stream));
     pop->cum_calls += pop->graph_n;
     if (pop->gb.lazy) {
