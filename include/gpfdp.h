@@ -345,8 +345,10 @@ int gp_set_graph_mode(gp_pop* pop, int on, uint64_t reserve_entries);
  * The graph holds the buffers the parents were in at its capture; parents
  * and children change places with every gp_crossover, reloads included in
  * the count, so gp_graph_launch returns GP_ESTATE after an odd number of
- * them (capture again, or breed one more generation).  The count r runs on
- * over gp_load_trees; a capture starts it at 0 again.
+ * them (capture again, or breed one more generation).  In fitness-first
+ * order it also returns GP_ESTATE after gp_load_trees until a generation of
+ * the new trees has drawn the plan that the replay starts with.  The count
+ * r runs on over gp_load_trees; a capture starts it at 0 again.
  */
 int gp_graph_capture(gp_pop* pop, uint32_t first_generation, uint32_t n_generations);
 int gp_graph_launch(gp_pop* pop);

@@ -1132,6 +1132,9 @@ int gp_graph_launch(gp_pop* pop) {
     if (pop->cur != pop->graph_cur)
         return fail(pop, GP_ESTATE, "an odd number of generations since the capture: parents and children have changed buffers "
                                     "(capture again)");
+    // and its first generation takes a plan drawn before the replay
+    if (pop->gb.lazy && !pop->have_next_plan)
+        return fail(pop, GP_ESTATE, "fitness-first mode: replay after a generation of the current trees");
     CK(cudaGraphLaunch(pop->gexec, pop->stream));
     pop->cum_calls += pop->graph_n;
     if (pop->gb.lazy) {

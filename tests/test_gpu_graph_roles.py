@@ -1,6 +1,7 @@
 """A captured graph between eager generations and reloads: its kernels hold the
 buffers of the capture, so a replay is refused while parents and children are
-in each other's buffers.  What is not refused equals the eager run bit for
+in each other's buffers, and in fitness-first order until the loaded trees
+have a plan of their own.  What is not refused equals the eager run bit for
 bit."""
 import numpy as np
 import pytest
@@ -57,3 +58,21 @@ def test_replay_after_an_odd_number_of_generations_is_refused():
     assert _state(pop) == want[5]
     pop.close()
 
+
+def test_replay_of_a_reloaded_fitness_first_population():
+    gp, w, pop = _pop(True)
+    pop.set_graph_mode(True)
+    pop.eval_full()
+    _generation(pop, 0)
+    pop.graph_capture(1, 2)
+    pop.graph_launch()
+    want = _state(pop)
+    pop.load_trees(w["ops"], w["off"])
+    pop.eval_full()
+    _refused(gp, pop)                                 # no plan of these trees yet
+    _generation(pop, 0)
+    _refused(gp, pop)                                 # the second generation outside the graph: buffers changed
+    pop.graph_capture(1, 2)
+    pop.graph_launch()
+    assert _state(pop) == want
+    pop.close()
