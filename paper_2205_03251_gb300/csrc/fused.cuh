@@ -23,8 +23,9 @@
 // window of W entries in shared memory slides over the stack from chunk to
 // chunk (entries below it in a global overflow area), and a chunk of 128
 // nodes whose depths span more than the window runs on the global area alone.
-// A malformed run (B negative somewhere, or not 1 at its start) is refused
-// before anything is executed that could leave the stack.
+// A malformed run has B below 1 after one of its nodes, or not 1 at its
+// start.  The first is found as the chunk with that node is decoded: chunks to
+// its right have run by then, that one does not, so nothing leaves the stack.
 #pragma once
 #include "interp.cuh"
 
@@ -159,10 +160,13 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     r.mx = b0 + max(max(d3, d2), max(d1, d0));
     r.mn = b0 + min(min(d3, d2), min(d1, d0));
     c.B += (int32_t)all >> 16;
+    // Well formed: one subtree or more complete after every node, so that each function finds two operands.  Words past
+    // the run's end have none yet; in the word that holds the end (at most three nodes of it) the next test says it all.
+    const int least = q + 4 <= (int32_t)e ? 1 : 0;
     // a function among the last two nodes of the run has no operands
     const int32_t last2 = (int32_t)e - 2 - q;
     const bool tail = (valid & f) != 0 && last2 < 4 && (valid & f & (last2 <= 0 ? 0xFFFFFFFFu : 0xFFFFFFFFu << (8 * last2))) != 0;
-    r.bad = __any_sync(FULL, r.mn < 0 || tail);
+    r.bad = __any_sync(FULL, r.mn < least || tail);
     // instruction indexes of the four bytes at once
     uint32_t idx, A;                     // index; the byte of the first operand
     uint32_t both, second = n2;          // f L L and f g L L with two table operands; the byte of the second
