@@ -444,8 +444,11 @@ int gp_set_profiling(gp_pop* pop, int on);
  * synchronises its stream before returning.  Returns GP_EINVAL for bad
  * arguments or a malformed tree, GP_ECAPACITY when a tree is empty, larger
  * than 1023 nodes or outside ops_bytes; *status_out (host, may be NULL) gets
- * the raw flags (1: size or bounds, 2: malformed tree, 4: no overflow
- * stack came free within the wait limit, returned as GP_ETIMEOUT).
+ * the raw flags (1: size or bounds, 2: malformed tree, 4: an overflow stack's
+ * turn did not change hands within the wait limit, returned as GP_ETIMEOUT;
+ * the number of trees waiting does not bring that about).  Trees deeper than
+ * a warp's stack window in shared memory (48 entries, 96 up to 32 cases) run
+ * on 64 warps at a time, the others on the whole GPU.
  */
 int gp_eval_small_noalloc(const uint8_t* d_ops, size_t ops_bytes, const uint64_t* d_off, uint32_t n_trees,
                           const float* d_x, const float* d_t, const float* d_consts, uint32_t n_cases,
