@@ -399,6 +399,7 @@ void launch_items(gp_pop* pop) {
 template <int K, int V>
 void launch_skeleton(gp_pop* pop) {
     // the flag words have room for 32 case blocks: more go in further launches
+    pop->launches += (pop->d.ncb - 1) / 32;
     for (uint32_t cb0 = 0; cb0 < pop->d.ncb; cb0 += 32) {
         const uint32_t n = pop->d.ncb - cb0 < 32u ? pop->d.ncb - cb0 : 32u;
         if (cb0) {
@@ -557,7 +558,7 @@ int run_full(gp_pop* pop) {
     const int gthreads = pop->grid_threads;
     CK(cudaMemsetAsync(d.q, 0, sizeof(uint32_t) * NQ, pop->stream));
     CK(cudaMemsetAsync(d.acc_ops, 0, 4 * sizeof(unsigned long long), pop->stream));
-    pop->launches = 15;
+    pop->launches = 15;                 // (launch_skeleton adds those beyond its first)
     pop->last_kind = 0;
     phase_begin(pop, PH_STRUCT);
     {
