@@ -1645,7 +1645,15 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, Ge
                     finish_level0();
                     if (fail) break;
                 }
-                if (ncm == nb) break;                      // nothing left to combine
+                if (ncm == nb) {                           // nothing left to combine: the child's root was replaced, or the
+                                                           // walk has stopped; else the links lead past the root, and
+                                                           // an inner subtree's value would pass for its fitness
+                    if (!stopped_w && c != 0) {
+                        if (lane == 0) set_error(d, ST_STRUCT, 9, i, c, ncm);
+                        fail = true;
+                    }
+                    break;
+                }
                 const uint32_t slot = ncm % ring;
                 __syncwarp();
                 const LevelDesc D = desc[slot];
