@@ -1475,13 +1475,25 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, Ge
     volatile uint32_t* vcnt = sc + 16 + WALK_RING;     // [WALK_RING] case blocks of the slot's sibling done
     const uint32_t nev = nw - 1;                       // sibling evaluators (warps 1..nw-1)
     const uint32_t ring = walk_ring(Cpad);
+    // counts of this launch: in 32 bits (in 64 more registers spilled), emptied into the 64-bit totals between children
+    // before they can wrap -- a child has at most 2^30 nodes, and none is counted twice in one count but the few below T
     uint32_t st_interp = 0, st_levels = 0, st_stopped = 0, st_pathops = 0;
+    auto tally = [&]() {
+        if (lane == 0) atomicAdd(&g.gstat[G_INTERP], (unsigned long long)st_interp);
+        if (tid == 0) {
+            atomicAdd(&g.gstat[G_LEVELS], (unsigned long long)st_levels);
+            atomicAdd(&g.gstat[G_STOPPED], (unsigned long long)st_stopped);
+            atomicAdd(&g.gstat[G_PATHOPS], (unsigned long long)st_pathops);
+        }
+        st_interp = st_levels = st_stopped = st_pathops = 0;
+    };
     auto cases = [&](uint32_t cb) {
         load_cases<K>(d, cb, ic.x);
         ic.lt = FxTable<K, V>::at(sm, cb);
     };
 
     for (;;) {
+        if ((st_interp | st_levels | st_stopped | st_pathops) >> 31) tally();
         if (tid == 0) sc[0] = atomicAdd(&d.q[wr.qctr], 1u);
         __syncthreads();
         const uint32_t qi = wr.q_lo + sc[0];
@@ -1866,12 +1878,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, Ge
         }
         __syncthreads();                     // nvs and the shared words are reused by the next child
     }
-    if (lane == 0) atomicAdd(&g.gstat[G_INTERP], (unsigned long long)st_interp);
-    if (tid == 0) {
-        atomicAdd(&g.gstat[G_LEVELS], (unsigned long long)st_levels);
-        atomicAdd(&g.gstat[G_STOPPED], (unsigned long long)st_stopped);
-        atomicAdd(&g.gstat[G_PATHOPS], (unsigned long long)st_pathops);
-    }
+    tally();
 }
 
 // ---- one-pass evaluation of children of at most ONEPASS_MAX nodes.
