@@ -111,6 +111,21 @@ __device__ __forceinline__ uint32_t find_segment(const uint32_t* off, uint32_t n
     return lo;
 }
 
+// An evaluator's place in a walk: item number = level * ncb + case block, of
+// which `ticket` holds the low 32 bits (a deep tree over many case blocks has
+// more items than that).  A new ticket is less than 2^32 items ahead of the
+// evaluator's last one, because the others can be no more than a ring of
+// levels ahead of the level it is at.
+struct WalkItem {
+    uint32_t ticket, level, cb;
+    __host__ __device__ void take(uint32_t t, uint32_t ncb) {
+        cb += t - ticket;
+        ticket = t;
+        level += cb / ncb;
+        cb %= ncb;
+    }
+};
+
 // Fitness of one value vector, whose case (Boolean: word) j is at(j):
 //   binary32: sum over the cases, in case order, of |v - t|, each step
 //             rounded to binary32;

@@ -1803,13 +1803,14 @@ __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, Ge
             // evaluators: each takes the next (level, case block) item in level order from a
             // shared counter and evaluates it once the level's descriptor is built, so a long
             // sibling holds up only the warp evaluating it
+            WalkItem item{0u, 0u, 0u};
             for (;;) {
                 uint32_t k = 0, cb = 0, fin = 0;
                 if (lane == 0) {
                     for (;;) {
-                        const uint32_t it = atomicAdd(const_cast<uint32_t*>(&sc[5]), 1u);
-                        k = it / ncb;
-                        cb = it % ncb;
+                        item.take(atomicAdd(const_cast<uint32_t*>(&sc[5]), 1u), ncb);
+                        k = item.level;
+                        cb = item.cb;
                         uint32_t spins = 0, tag = 0;
                         for (;;) {
                             if (sc[8]) { fin = 1; break; }                  // the combination is over
