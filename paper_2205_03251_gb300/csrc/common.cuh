@@ -74,7 +74,6 @@ struct DevPop {
     unsigned long long* acc_ops;   // [4] actual-op counters
 };
 
-__device__ __forceinline__ uint32_t warp_bcast(uint32_t v, int src) { return __shfl_sync(FULL, v, src); }
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 // In graph mode the cache arrays are never regrown: a kernel that finds the
@@ -126,38 +125,17 @@ struct WalkItem {
     }
 };
 
-// Fitness of one value vector, whose case (Boolean: word) j is at(j):
+// Fitness of one value vector, whose case (Boolean: word) j is at(j), by the
+// whole warp (all 32 lanes call it; every lane returns the fitness):
 //   binary32: sum over the cases, in case order, of |v - t|, each step
-//             rounded to binary32;
+//             rounded to binary32: the lanes fetch and form the terms of 32
+//             cases at a time, and every lane adds them in case order from
+//             shuffles;
 //   Boolean:  the number of wrong cases, popcount(v ^ target) summed over
 //             the words;
 //   integer:  sum of |v - t| exact in 64-bit integers, rounded once to
 //             binary32.
-template <typename F>
-__device__ __forceinline__ float fitness_of(const DevPop& d, F at) {
-    if (d.vkind == VB) {
-        uint32_t e = 0;
-        for (uint32_t j = 0; j < d.C; ++j) e += __popc(__float_as_uint(at(j)) ^ __float_as_uint(d.t[j]));
-        return (float)e;
-    }
-    if (d.vkind == VI) {
-        long long s = 0;
-        for (uint32_t j = 0; j < d.C; ++j) {
-            const long long e = (long long)__float_as_int(at(j)) - (long long)__float_as_int(d.t[j]);
-            s += e < 0 ? -e : e;
-        }
-        return __ll2float_rn(s);
-    }
-    float f = 0.0f;
-    for (uint32_t j = 0; j < d.C; ++j) f = __fadd_rn(f, fabsf(__fsub_rn(at(j), d.t[j])));
-    return f;
-}
-
-// fitness_of with the whole warp (all 32 lanes call it; every lane returns
-// the fitness): the lanes fetch and form the terms of 32 cases at a time in
-// parallel, and every lane adds them in case order from shuffles, so the
-// binary32 sum is rounded in the same order and has the same bits; the
-// Boolean and integer sums are exact, so their order does not matter.
+// The Boolean and integer sums are exact, so their order does not matter.
 template <typename F>
 __device__ __forceinline__ float fitness_warp(const DevPop& d, F at) {
     const uint32_t lane = threadIdx.x & 31u;

@@ -998,11 +998,7 @@ __device__ __forceinline__ void load_blk(const float* row, uint32_t cb, float (&
 }
 
 
-// Shared-memory layout of one walk team (a CTA of nw warps working on one
-// child): constant tables, the small-ancestor lists, the level descriptors
-// of a batch, the running value vectors of the child and of the mother,
-// the siblings' vectors of a batch, a few broadcast words, then per warp an
-// interpreter stack and two staging buffers.
+// A level of the walk: an ancestor of the crossover point and its sibling.
 struct __align__(16) LevelDesc {
     uint32_t ss, se;            // sibling range in the child
     uint32_t p, pend;           // ancestor, its end in the child
@@ -1024,7 +1020,12 @@ struct __align__(16) LevelDesc {
 // levels in flight: fewer when value vectors are long
 __host__ __device__ inline uint32_t walk_ring(uint32_t Cpad) { return Cpad <= 128 ? 32u : Cpad <= 256 ? 8u : 4u; }
 
-// (tab: bytes of the interpreter's leaf table, first so that its addresses fit 16 bits)
+// Shared-memory layout of one walk team (a CTA of nw warps working on one
+// child): the interpreter's leaf table (tab bytes, first so that its addresses
+// fit 16 bits), the small-ancestor lists, the ring of level descriptors, the
+// running value vectors of the child and of the mother, the siblings' vectors
+// of the ring, a few broadcast words, then per warp a stack window and the
+// instruction list of a chunk.
 template <int K>
 struct TeamLayout {
     uint32_t anc, ancg, lvl, desc, nv, ov, sv, sc, warp0, warp_bytes, total;
@@ -2554,7 +2555,7 @@ __global__ void __cluster_dims__(FREE_CTAS, 1, 1) __launch_bounds__(FREE_THREADS
 // New values of the children's cache (walk records): each record that
 // became an entry takes the free slot of its rank; one warp per record,
 // lanes over cases.
-__global__ void k_copy_values(DevPop d, GenBufs g, CacheView par) {
+__global__ void k_copy_values(DevPop d, GenBufs g) {
     if (halted(d)) return;
     const uint32_t ne = d.e_off[d.P];
     if (ne > d.Ecap) return;
@@ -2573,7 +2574,6 @@ __global__ void k_copy_values(DevPop d, GenBufs g, CacheView par) {
         for (uint32_t k = lane; k < d.Cpad; k += 32) dp[k] = __ldcg(sp + k);
         if (lane == 0) d.e_slot[x] = sl;
     }
-    (void)par;
 }
 
 // equivalent-op count of the children (every opcode on every case)

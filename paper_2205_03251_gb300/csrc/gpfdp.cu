@@ -165,12 +165,6 @@ int dalloc(gp_pop* pop, T** ptr, size_t count) {
     return GP_OK;
 }
 
-#define DA(ptr, n)                                   \
-    do {                                             \
-        int r_ = dalloc(pop, &(ptr), (size_t)(n));   \
-        if (r_) return r_;                           \
-    } while (0)
-
 void phase_begin(gp_pop* pop, int ph, cudaStream_t st) {
     if (!pop->profiling) return;
     if (pop->capturing) {
@@ -1716,7 +1710,7 @@ int gen_incremental(gp_pop* pop) {
     k_child_sizes<<<(d.P + 255) / 256, 256, 0, pop->side3>>>(d, g);
     CK(cudaEventRecord(pop->xjoin_ev[1], pop->side3));
     k_free_find<<<FREE_CTAS, FREE_THREADS, 0, pop->stream>>>(d, g);
-    k_copy_values<<<pop->nsm * 16, 256, 0, pop->stream>>>(d, g, par);
+    k_copy_values<<<pop->nsm * 16, 256, 0, pop->stream>>>(d, g);
     k_check_slots<<<gt, 256, 0, pop->stream>>>(d);
     CK(cudaStreamWaitEvent(pop->stream, pop->xjoin_ev[1], 0));
     CK(cudaStreamWaitEvent(pop->stream, pop->join_ev, 0));
