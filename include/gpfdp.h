@@ -347,8 +347,11 @@ int gp_set_graph_mode(gp_pop* pop, int on, uint64_t reserve_entries);
  * the count, so gp_graph_launch returns GP_ESTATE after an odd number of
  * them (capture again, or breed one more generation).  In fitness-first
  * order it also returns GP_ESTATE after gp_load_trees until a generation of
- * the new trees has drawn the plan that the replay starts with.  The count
- * r runs on over gp_load_trees; a capture starts it at 0 again.
+ * the new trees has drawn the plan that the replay starts with.
+ * The count r runs on over gp_load_trees, and the generation numbers with it
+ * (in fitness-first order from the second generation of the replay on: the
+ * first follows the plan already drawn); to breed a reloaded population with
+ * the numbers from first_generation on, capture again, which starts r at 0.
  */
 int gp_graph_capture(gp_pop* pop, uint32_t first_generation, uint32_t n_generations);
 int gp_graph_launch(gp_pop* pop);

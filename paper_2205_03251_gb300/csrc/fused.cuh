@@ -161,12 +161,12 @@ __device__ __forceinline__ FxChunk fx_decode(FxCarry& c, uint32_t fl_word, int32
     r.mn = b0 + min(min(d3, d2), min(d1, d0));
     c.B += (int32_t)all >> 16;
     // Well formed: one subtree or more complete after every node, so that each function finds two operands.  Words past
-    // the run's end have none yet; in the word that holds the end (at most three nodes of it) the next test says it all.
-    const int least = q + 4 <= (int32_t)e ? 1 : 0;
+    // the run's end have none yet, nor need the word that holds the end (at most three nodes of it; its top byte is not
+    // valid): there the next test says it all.
     // a function among the last two nodes of the run has no operands
     const int32_t last2 = (int32_t)e - 2 - q;
     const bool tail = (valid & f) != 0 && last2 < 4 && (valid & f & (last2 <= 0 ? 0xFFFFFFFFu : 0xFFFFFFFFu << (8 * last2))) != 0;
-    r.bad = __any_sync(FULL, r.mn < least || tail);
+    r.bad = __any_sync(FULL, r.mn < (int32_t)(valid >> 31) || tail);
     // instruction indexes of the four bytes at once
     uint32_t idx, A;                     // index; the byte of the first operand
     uint32_t both, second = n2;          // f L L and f g L L with two table operands; the byte of the second
