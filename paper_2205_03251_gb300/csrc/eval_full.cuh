@@ -64,12 +64,15 @@ struct ItemsLayout {
 
 // Persistent warps over (item, case block) units.  The next unit's index,
 // descriptor and first words are fetched while the current one is evaluated.
-// Bound by the indirect branch of each instruction (about 24 cycles of an
-// SM quarter, whatever it branches to; 0.53 instructions a node on grafted
-// trees), which 16 warps per SM saturate.  500 grafted trees of ~1e6 nodes x
-// 48 cases: 14.4 ms node by node, 6.6 ms now; 2,001 uneven integer trees 1.59
-// -> 0.95 ms; 600 uneven trees x 1,000 cases 5.57 -> 3.2 ms.  The words are
-// read straight from the tree, a chunk ahead (no staged copy).
+// Grafted trees: bound by the indirect branch of each instruction (about 24
+// cycles of an SM quarter, whatever it branches to; 0.53 instructions a node),
+// which 16 warps per SM saturate.  Uneven trees: bound by the units -- half of
+// their items are one leaf, 94 % fit a chunk, and each costs a place in the
+// queue, a descriptor, a decode and a value vector whatever its length.  500
+// grafted trees of ~1e6 nodes x 48 cases: 12.6 ms node by node, 6.7 ms now;
+// 2,001 uneven integer trees 1.57 -> 0.94 ms; 600 uneven trees x 1,000 cases
+// 4.98 -> 2.13 ms.  The words are read straight from the tree, a chunk ahead
+// (no staged copy).
 template <int K, int V>
 __global__ void __launch_bounds__(GP_WARPS * 32, K == 4 ? 3 : V == VF ? 4 : 5) k_eval_items(DevPop d) {
     if (halted(d)) return;
@@ -156,8 +159,8 @@ __global__ void __launch_bounds__(GP_WARPS * 32, K == 4 ? 3 : V == VF ? 4 : 5) k
 // No warp waits.  Bound by latency along a tree's longest chain; every chain
 // and case block runs at once, where a warp per tree took the chains and the
 // case blocks one after another: 500 grafted trees of ~1e6 nodes x 48 cases
-// 1.10 -> 0.43 ms, 1,500 uneven trees over the 11-multiplexer 1.06 -> 0.38 ms,
-// 600 uneven trees x 1,000 cases 14.2 -> 0.67 ms.  cb0, ncbp: the case blocks
+// 1.03 -> 0.32 ms, 1,500 uneven trees over the 11-multiplexer 1.16 -> 0.52 ms,
+// 600 uneven trees x 1,000 cases 13.4 -> 0.56 ms.  cb0, ncbp: the case blocks
 // of this launch (at most 32, the bits of a flag word).
 #define SKB 8
 #define SK_WARPS 4

@@ -1440,11 +1440,12 @@ struct WalkRange {
 // interpreted nodes takes a team about 200 us, a third of a warp's cycles
 // waiting for instructions (one warp of a team combines, the others run the
 // interpreter).  Two forms: MAXT 128 keeps 5 teams of 4 warps on an SM (96
-// registers, some spilled) for populations whose children queue for teams;
-// MAXT 512 keeps its registers (4 teams of 4 warps) for populations whose
-// longest walk counts, and for larger teams.  4,096 uneven trees 3.4 -> 1.5 ms
-// (1.65 with the second form), 500 grafted trees of 1e6 nodes 0.30 -> 0.17 ms
-// (0.19 with the first).
+// registers; four cases per lane spill some) for populations whose children
+// queue for teams; MAXT 512 keeps its registers (4 teams of 4 warps) for
+// populations whose longest walk counts, and for larger teams.  The fourth
+// generation of 4,096 uneven trees 1.91 -> 0.91 ms (0.97 with the second
+// form), of 500 grafted trees of 1e6 nodes 0.24 -> 0.15 ms (0.16 with the
+// first).
 template <int K, int V, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 128 ? 5 : 1) k_walk(DevPop d, GenBufs g, CacheView par, uint32_t nw,
                                                            WalkRange wr) {
@@ -2131,8 +2132,8 @@ __global__ void __launch_bounds__(ONEPASS_WARPS * 32) k_onepass_plan(DevPop d, G
 
 // Bound by the interpreter's indirect branches and, for small children, by
 // the chain of loads before the first word.  4,096 uneven trees x 48 cases
-// 0.58 -> 0.25 ms, 2,048 over the 6-multiplexer 0.51 -> 0.22 ms, 500 ramped
-// trees 67 -> 33 us against the interpreter that took node by node from
+// 0.58 -> 0.28 ms, 2,048 over the 6-multiplexer 0.46 -> 0.24 ms, 500 ramped
+// trees 58 -> 28 us against the interpreter that took node by node from
 // pieces staged in shared memory.
 template <int K, int V>
 __global__ void __launch_bounds__(OP_EVAL_WARPS * 32, 3) k_onepass_eval(DevPop d, GenBufs g) {
@@ -2494,9 +2495,9 @@ __global__ void __launch_bounds__(256) k_merge_write(DevPop d, GenBufs g, CacheV
 // first slot, FREE_PER slots to a thread (131,072 a step), until it has found
 // them; the CTAs' counts go round through distributed shared memory.  The pool
 // has at least as many free slots as there are records besides the entries'
-// own, usually half of it, so one or two steps do, where counting all tiles
-// of the pool, their prefix and the list took three launches (22 us at 4
-// million slots).
+// own, usually half of it, so one or two steps do: 11 us on 500 trees of 1e6
+// nodes, where counting all tiles of the pool, their prefix and the list took
+// three launches of 22 us together.
 #define FREE_CTAS 8
 #define FREE_THREADS 512
 #define FREE_PER 32

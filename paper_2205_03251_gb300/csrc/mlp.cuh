@@ -286,8 +286,8 @@ __global__ void k_mlp_init(MlpBufs b, uint64_t seed) {
 // ranks: the rank of key i is the number of keys that come before it, so
 // order[rank(i)] = i.  A CTA ranks RANK_KEYS keys, its eight warps a share of
 // the n comparisons each (four keys a load), so that the n^2 comparisons
-// spread over the GPU and every rank is complete in one launch: 4,096 keys 62
-// -> 12 us, 500 keys 10 -> 4 us against a thread per key.
+// spread over the GPU and every rank is complete in one launch: 4,096 keys 20
+// -> 12 us (two launches before), 500 keys 10 -> 4 us against a thread per key.
 __device__ __forceinline__ float sort_key(const float* key, uint32_t i) {
     const float k = key[i];
     return isnan(k) ? -INFINITY : k;

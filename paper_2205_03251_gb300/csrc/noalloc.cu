@@ -73,8 +73,8 @@ struct NaLayout {
 // case order), or, when there are fewer trees than CTAs, a CTA per tree with
 // its warps on the case blocks.  The first trees go round the CTAs, so that a
 // few trees run on as many SMs; the others come from the counter.  3,000
-// uneven trees of up to 1,023 nodes x 100 cases: 2,591 us with 64 warps on
-// the whole chip, 133 us with 16 on each SM.
+// uneven trees of up to 1,023 nodes x 100 cases: 2,150 us with 64 warps on
+// the whole chip, 129 us with 16 on each SM.
 template <int K>
 __global__ void __launch_bounds__(NA_WARPS * 32) k_eval_small_noalloc(NaArgs a, uint32_t by_cta) {
     extern __shared__ __align__(16) unsigned char smem_raw[];

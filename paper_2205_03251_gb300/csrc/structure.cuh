@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(FLAG_WARPS * 32) k_unit_flags(DevPop d, Struct
 // window.  A warp takes up to FLAG_SPAN blocks in a row and computes each block's
 // chunk sums and maxima once (they serve as the next block's too).  Bound by
 // integer instructions; 0.5 GB of opcodes at a threshold of 1,024: 1.19 ms
-// with the window maxima of every position through shared memory, 0.37 ms.
+// with the window maxima of every position through shared memory, 0.35 ms.
 #define FLAG_SPAN 8
 __global__ void __launch_bounds__(FLAG_WARPS * 32) k_unit_flags_wide(DevPop d, StructBufs sb) {
     const int lane = lane_id();
