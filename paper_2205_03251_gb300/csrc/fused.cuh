@@ -499,33 +499,35 @@ __device__ __forceinline__ void fx_exec_global(uint32_t& ip, float (&a)[K], uint
         const uint32_t idx = lds_u32(ip), y = lds_u32(ip + 12);
         if (idx == FX_EXIT) break;
         float l[K], r[K];
-        if (V == VB && idx >= 32u) {
-            leaf(y & 0xFFFFu, true, l);
-            leaf(y >> 16, true, r);
-            apply_vec<K, V>((idx >> 2) & 3u, l, r);
-            apply_vec<K, V>((idx - 32u) >> 4, l, a);
+        // What a chunk of great depths mostly holds comes first: leaves that wait, functions that take two values.  (A lone
+        // warp pays for each branch: 3,000 left combs of 1,023 nodes x 100 cases 15.4 -> 13.9 ms.)
+        if (idx >= 28u) {
+            if (V == VB && idx >= 32u) {
+                leaf(y & 0xFFFFu, true, l);
+                leaf(y >> 16, true, r);
+                apply_vec<K, V>((idx >> 2) & 3u, l, r);
+                apply_vec<K, V>((idx - 32u) >> 4, l, a);
+            } else {
+                push();
+                leaf(y, idx & 1u, l);
+            }
 #pragma unroll
             for (int k = 0; k < K; ++k) a[k] = l[k];
-        } else if (idx < 16u) {
-            const bool ca = idx & 2u, cb = idx & 1u;
-            push();
-            leaf(ca && cb ? y & 0xFFFFu : y, ca, l);
-            leaf(ca && cb ? y >> 16 : y, cb, r);
-            apply_vec<K, V>(idx >> 2, l, r);
-#pragma unroll
-            for (int k = 0; k < K; ++k) a[k] = l[k];
-        } else if (idx < 24u) {
-            leaf(y, idx & 1u, l);
-            apply_vec<K, V>((idx - 16u) >> 1, l, a);
-#pragma unroll
-            for (int k = 0; k < K; ++k) a[k] = l[k];
-        } else if (idx < 28u) {
+        } else if (idx >= 24u) {
             --dep;
             vload<K>(g + (size_t)dep * 32 * K, r);
             apply_vec<K, V>(idx - 24u, a, r);
         } else {
-            push();
-            leaf(y, idx & 1u, l);
+            if (idx < 16u) {
+                const bool ca = idx & 2u, cb = idx & 1u;
+                push();
+                leaf(ca && cb ? y & 0xFFFFu : y, ca, l);
+                leaf(ca && cb ? y >> 16 : y, cb, r);
+                apply_vec<K, V>(idx >> 2, l, r);
+            } else {
+                leaf(y, idx & 1u, l);
+                apply_vec<K, V>((idx - 16u) >> 1, l, a);
+            }
 #pragma unroll
             for (int k = 0; k < K; ++k) a[k] = l[k];
         }

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(NA_WARPS * 32) k_eval_small_noalloc(NaArgs a, 
     // counted anew with each turn.  (A free stack for whoever takes it first
     // drew thousands of warps to one word, and without an order one of them
     // could miss every stack.  20,000 trees of 121 nodes and depth 61 x 100
-    // cases 15.2 -> 12.4 ms.)
+    // cases 14.0 -> 10.7 ms.)
     auto need = [&]() -> bool {
         if (held >= 0) return true;
         int got = -1;
