@@ -159,8 +159,8 @@ __global__ void __launch_bounds__(GP_WARPS * 32, K == 4 ? 3 : V == VF ? 4 : 5) k
 // No warp waits.  Bound by latency along a tree's longest chain; every chain
 // and case block runs at once, where a warp per tree took the chains and the
 // case blocks one after another: 500 grafted trees of ~1e6 nodes x 48 cases
-// 1.03 -> 0.32 ms, 1,500 uneven trees over the 11-multiplexer 1.16 -> 0.52 ms,
-// 600 uneven trees x 1,000 cases 13.4 -> 0.56 ms.  cb0, ncbp: the case blocks
+// 1.03 -> 0.32 ms, 1,500 uneven trees over the 11-multiplexer 1.16 -> 0.44 ms,
+// 600 uneven trees x 1,000 cases 13.4 -> 0.51 ms.  cb0, ncbp: the case blocks
 // of this launch (at most 32, the bits of a flag word).
 #define SKB 8
 #define SK_WARPS 4
